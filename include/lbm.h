@@ -324,8 +324,10 @@ int lbm_get_timing(lbm_ctx* ctx, double* ms_by_kind /* [3] */, long long* launch
  * 8-9 the row march staged by bulk tensor copies (TMA; on lattices whose
  * rows are not a multiple of 16 bytes they run the per-thread-copy march of
  * the same tile shape, variants 2 and 0).
- * D3Q27: 0-2 fused halo tiles, 3-4 the staged two-pass form, 5 the staged
- * form with the gradient inputs computed in a pass of their own.  Every form
+ * D3Q27: every form is the two-pass step split by lattice (one warp per
+ * lattice of 32 nodes); the indices select the registers a thread may use
+ * (0: one resident block per SM, 1: two, 2: three, 3: four; 4 and 5 the
+ * default).  Every form
  * computes the same step (the gradient stencil is summed in different
  * orders, so the forms agree to rounding).  New contexts use variant 5 in
  * 3-D and, in 2-D, variant 8 on lattices of at least 2^18 nodes without a

@@ -16,10 +16,11 @@ template <class To, class From>
 void params_cast(const Params<From>& s, Params<To>& d) {
   d.nx = s.nx; d.ny = s.ny; d.nz = s.nz; d.N = s.N;
   d.bc_lo = s.bc_lo; d.bc_hi = s.bc_hi; d.knudsen = s.knudsen;
-  d.RU = To(s.RU);
+  d.RU = To(s.RU); d.Kc = To(s.Kc);
   for (int a = 0; a < MMAX; ++a) {
     d.m[a] = To(s.m[a]); d.Ra[a] = To(s.Ra[a]); d.muref[a] = To(s.muref[a]);
     d.cvR[a] = To(s.cvR[a]); d.U0[a] = To(s.U0[a]); d.knc[a] = To(s.knc[a]);
+    d.inv_m[a] = To(s.inv_m[a]); d.mum[a] = To(s.mum[a]);
     for (int b = 0; b < MMAX; ++b) d.invDmm[a][b] = To(s.invDmm[a][b]);
     d.rho_in[0][a] = To(s.rho_in[0][a]); d.rho_in[1][a] = To(s.rho_in[1][a]);
   }

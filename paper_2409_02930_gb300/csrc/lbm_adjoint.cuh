@@ -51,32 +51,13 @@ struct AdjArgs {
   int* status;
 };
 
-// Streamed populations of node n (base type) with the boundary rules.
-template <class B, int D, int M, bool EN>
-LBM_HD void pull_node(const Params<B>& p, const InletTables<B>& it, const B* f, const B* phi, int x, int y, int z,
-                      B* P) {
-  constexpr int Q = Lat<D>::Q, L = n_lat<D, M, EN>();
-  Site<B, D> st;
-  st.init(p, x, y, z);
-  Ghost<B, D> gh;
-  gh.side = -1;
-  if (st.has_ghost()) ghost_velocity<B, D, M>(p, f, phi, x, y, z, gh);
-  for_each_dir<D>([&](int i, int cx, int cy, int cz) {
-    const int h = st.source(cx, cy, cz);
-#pragma unroll
-    for (int l = 0; l < L; ++l) P[l * Q + i] = pull_rt<B, D, M, EN>(p, it, f, gh, st.n, h, l, i, cx, cy, cz);
-  });
-}
-
 // Streamed populations of the node as dual numbers with zero derivative: the
 // node update's dependence on them is split into the moments (seeded) and
 // the direct relaxation term (coefficient returned by collide_gen).
 template <class B, int K, int D, int M, bool EN>
 struct PlainPull {
   const B* P;
-  static constexpr bool kUnroll = false;
-  LBM_HD int prep(int, int, int) const { return 0; }
-  LBM_HD Dual<B, K> get(int, int l, int i, int, int, int) const { return Dual<B, K>(P[l * Lat<D>::Q + i]); }
+  LBM_HD Dual<B, K> get(int l, int i) const { return Dual<B, K>(P[l * Lat<D>::Q + i]); }
 };
 
 // Moments seeded in the dual lanes [first, first + K) of a running index
@@ -114,15 +95,6 @@ LBM_HD void seed_moments(const Moments<B, D, M, EN, true>& m0, int first, Moment
 template <int D, int M>
 LBM_HD constexpr int n_mom() { return M + M * D + 1 + D + D * D + 1 + D; }
 
-// Base-type puller over the node's streamed populations.
-template <class B, int D>
-struct BasePull {
-  const B* P;
-  static constexpr bool kUnroll = false;
-  LBM_HD int prep(int, int, int) const { return 0; }
-  LBM_HD B get(int, int l, int i, int, int, int) const { return P[l * Lat<D>::Q + i]; }
-};
-
 // Node update: lambda^{n+1}(x)^T dC / d(lambda, phi(x), G(x), P(x)).  The
 // populations enter the node update through the moments and through the
 // direct relaxation term: dC_{l,i}/dP_{l,j} = coef_l delta_ij for i, j not
@@ -146,7 +118,7 @@ __global__ void __launch_bounds__(128) k_adj_collide(Params<B> p, InletTables<B>
   B P[LQ];
   pull_node<B, D, M, EN>(p, it, a.f, a.phi, x, y, z, P);
   Moments<B, D, M, EN, true> m0;
-  moments_gen<B, D, M, EN, true>(BasePull<B, D>{P}, m0);
+  moments_gen<B, D, M, EN, true>(ArrayPull<B, D>{P}, m0);
   Grad<B, D, M, EN> g0;
   const B* __restrict__ mac = a.mac;
   g0.compute(p, x, y, z, [&](int k, int nb) { return mac[(size_t)k * N + nb]; });
@@ -184,7 +156,7 @@ __global__ void __launch_bounds__(128) k_adj_collide(Params<B> p, InletTables<B>
     State<T, D, M> s;
     s.template from_moments<EN, true>(pp, mo, phid, T(Tf));
     T out[LQ], cf[L];
-    collide_gen<T, D, M, EN, PlainPull<B, K, D, M, EN>, false, true>(pp, pf, 0, mo, s, gd, out, a.status, nullptr, cf);
+    collide_gen<T, D, M, EN, PlainPull<B, K, D, M, EN>, true>(pp, pf, 0, mo, s, gd, out, a.status, cf);
 #pragma unroll
     for (int l = 0; l < L; ++l) coef[l] = cf[l].v;
 #pragma unroll
@@ -208,7 +180,9 @@ __global__ void __launch_bounds__(128) k_adj_collide(Params<B> p, InletTables<B>
   const B* mb_Pt = mbar + M + M * D + 1 + D;
   const B mb_sg = mbar[M + M * D + 1 + D + D * D];
   const B* mb_q = mbar + M + M * D + 1 + D + D * D + 1;
-  for_each_dir<D>([&](int i, int cx, int cy, int cz) {
+  Unroll<0, Q>::run([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    constexpr int cx = c_of<D>(i, 0), cy = c_of<D>(i, 1), cz = c_of<D>(i, 2);
     const int cc[3] = {cx, cy, cz};
 #pragma unroll
     for (int l = 0; l < L; ++l) {
@@ -310,7 +284,9 @@ __global__ void __launch_bounds__(128) k_adj_macro(Params<B> p, InletTables<B> i
   for (int k = 0; k < M; ++k) sa[k] = B(0);
 #pragma unroll
   for (int b = 0; b < D; ++b) jf[b] = B(0);
-  for_each_dir<D>([&](int i, int cx, int cy, int cz) {
+  Unroll<0, Q>::run([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    constexpr int cx = c_of<D>(i, 0), cy = c_of<D>(i, 1), cz = c_of<D>(i, 2);
     const int cc[3] = {cx, cy, cz};
 #pragma unroll
     for (int k = 0; k < M; ++k) sa[k] += P[k * Q + i];
@@ -343,7 +319,7 @@ __global__ void __launch_bounds__(128) k_adj_macro(Params<B> p, InletTables<B> i
     T m[NMAC];
 #pragma unroll
     for (int b = 0; b < D; ++b) {
-      m[b] = s.u[b];
+      m[b] = s.u(b);
       m[D + b] = s.Pi(b);
     }
     if (EN) {
@@ -360,7 +336,9 @@ __global__ void __launch_bounds__(128) k_adj_macro(Params<B> p, InletTables<B> i
     }
   }
   // d(moments)/dP: species sums, momentum-lattice mass and momentum, energy sum
-  for_each_dir<D>([&](int i, int cx, int cy, int cz) {
+  Unroll<0, Q>::run([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    constexpr int cx = c_of<D>(i, 0), cy = c_of<D>(i, 1), cz = c_of<D>(i, 2);
     const int cc[3] = {cx, cy, cz};
 #pragma unroll
     for (int k = 0; k < M; ++k) a.Pbar[(size_t)(k * Q + i) * N + n] += bar[k];
@@ -380,7 +358,7 @@ template <class B, int D, int M, bool EN, int K>
 __global__ void __launch_bounds__(128) k_adj_ghost(Params<B> p, InletTables<B> it, AdjArgs<B> a,
                                                    const __grid_constant__ AdjParams<B, K> ap) {
   using T = Dual<B, K>;
-  constexpr int Q = Lat<D>::Q, L = n_lat<D, M, EN>();
+  constexpr int Q = Lat<D>::Q;
   static_assert(D + 3 <= K, "ghost directions exceed the dual lanes");
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= p.ny * p.nz) return;
@@ -404,7 +382,9 @@ __global__ void __launch_bounds__(128) k_adj_ghost(Params<B> p, InletTables<B> i
     B s0 = B(0), j[D];
 #pragma unroll
     for (int b = 0; b < D; ++b) j[b] = B(0);
-    for_each_dir<D>([&](int i, int cx, int cy, int cz) {
+    Unroll<0, Q>::run([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    constexpr int cx = c_of<D>(i, 0), cy = c_of<D>(i, 1), cz = c_of<D>(i, 2);
       const B f = a.f[(size_t)(M * Q + i) * N + sa.source(cx, cy, cz)];
       const int cc[3] = {cx, cy, cz};
       s0 += f;
@@ -428,22 +408,19 @@ __global__ void __launch_bounds__(128) k_adj_ghost(Params<B> p, InletTables<B> i
 #pragma unroll
     for (int b = 0; b < D; ++b) gh.u[b] = jd[b] / rho_f;
     gh.phi = seeded(a.phi[nb], D + 2);
-    Site<B, D> sb;
-    sb.init(p, xb, y, z);
     B acc[D + 3];
 #pragma unroll
     for (int k = 0; k < D + 3; ++k) acc[k] = B(0);
-    for_each_dir<D>([&](int i, int cx, int cy, int cz) {
-      if (sb.source(cx, cy, cz) != SRC_GHOST) return;
+    const int into = side == 0 ? 1 : -1;               // c_x of the missing directions
+    ghost_face<T, D, M, EN>(ap.pz, itd, gh, [&](int l, int cy, int cz, const T& g) {
+      const int i = (into + 1) + 3 * (cy + 1) + ((D == 3) ? 9 * (cz + 1) : 0);
+      const B pb = a.Pbar[(size_t)(l * Q + i) * N + nb];
 #pragma unroll
-      for (int l = 0; l < L; ++l) {
-        const T g = pull_rt<T, D, M, EN>(ap.pz, itd, (const T*)nullptr, gh, nb, SRC_GHOST, l, i, cx, cy, cz);
-        const B pb = a.Pbar[(size_t)(l * Q + i) * N + nb];
-#pragma unroll
-        for (int k = 0; k < D + 3; ++k) acc[k] += pb * g.d[k];
-      }
+      for (int k = 0; k < D + 3; ++k) acc[k] += pb * g.d[k];
     });
-    for_each_dir<D>([&](int i, int cx, int cy, int cz) {
+    Unroll<0, Q>::run([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    constexpr int cx = c_of<D>(i, 0), cy = c_of<D>(i, 1), cz = c_of<D>(i, 2);
       const int cc[3] = {cx, cy, cz};
       B v = acc[0];
 #pragma unroll

@@ -10,7 +10,6 @@
 // tiles inside one case.
 #pragma once
 
-#include "lbm_kernels.cuh"
 #include "lbm_staged.cuh"
 
 namespace lbm {

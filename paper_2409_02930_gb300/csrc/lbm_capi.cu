@@ -43,10 +43,11 @@ template <class R>
 void convert_params(const lbm::Params<double>& d, lbm::Params<R>& r) {
   r.nx = d.nx; r.ny = d.ny; r.nz = d.nz; r.N = d.N;
   r.bc_lo = d.bc_lo; r.bc_hi = d.bc_hi; r.knudsen = d.knudsen;
-  r.RU = (R)d.RU;
+  r.RU = (R)d.RU; r.Kc = (R)d.Kc;
   for (int a = 0; a < lbm::MMAX; ++a) {
     r.m[a] = (R)d.m[a]; r.Ra[a] = (R)d.Ra[a]; r.muref[a] = (R)d.muref[a];
     r.cvR[a] = (R)d.cvR[a]; r.U0[a] = (R)d.U0[a]; r.knc[a] = (R)d.knc[a];
+    r.inv_m[a] = (R)d.inv_m[a]; r.mum[a] = (R)d.mum[a];
     for (int b = 0; b < lbm::MMAX; ++b) r.invDmm[a][b] = (R)d.invDmm[a][b];
     r.rho_in[0][a] = (R)d.rho_in[0][a]; r.rho_in[1][a] = (R)d.rho_in[1][a];
   }
@@ -147,6 +148,8 @@ void make_params(const lbm_config* c, Params<double>& p, InletTables<double>& it
   for (int a = 0; a < M; ++a) {
     p.Ra[a] = p.RU / p.m[a];
     p.muref[a] = c->mu_ref[a] / (cvel * c->dx);
+    p.inv_m[a] = 1.0 / p.m[a];
+    p.mum[a] = p.muref[a] / p.m[a];
     p.cvR[a] = c->cv_factor[a] * p.Ra[a];
     p.U0[a] = c->U0[a] / c2;
     for (int b = 0; b < M; ++b)
@@ -161,6 +164,7 @@ void make_params(const lbm_config* c, Params<double>& p, InletTables<double>& it
   p.T_thermo = c->T_thermo;
   p.inv_T_ref = 1.0 / c->T_ref;
   p.Pref = c->P_ref / c2;
+  p.Kc = p.RU * p.RU * c->T_ref * std::sqrt(c->T_ref) / p.Pref;
   p.kappa_thr = c->kappa_threshold > 0 ? c->kappa_threshold : 1e3;
   p.wait_limit = kDefaultWaitLimit;
   std::memset(&it, 0, sizeof(it));
@@ -313,9 +317,9 @@ int lbm_create(lbm_ctx** out, const lbm_config* c) {
   const size_t rs = real_size(x);
   const size_t pop_bytes = (size_t)x->L * x->Q * N * rs;
   void* ptrs[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  // macro scratch: u, Pi, Y_a, and in 3-D the gradient inputs of the staged
-  // form with a gradient pass (1 + D + M D more fields)
-  const size_t mac_fields = (size_t)(2 * x->D + M) + (x->D == 3 ? (size_t)(1 + x->D + M * x->D) : 0);
+  // macro scratch: u, Pi, Y_a, and with a surface mechanism the species sums
+  // and temperatures that its source reads (M + 1 more fields)
+  const size_t mac_fields = (size_t)(2 * x->D + M) + (c->S > 0 ? (size_t)(M + 1) : 0);
   size_t sizes[6] = {pop_bytes, pop_bytes, N * rs, N * rs, mac_fields * N * rs, 64};
   for (int k = 0; k < 6; ++k) {
     e = cudaMalloc(&ptrs[k], sizes[k]);

@@ -48,6 +48,10 @@ struct Params {
   R cvR[MMAX];                // C_v,a = cv_factor_a R_a
   R U0[MMAX];
   R knc[MMAX];                // 1/tau^k_a = knc_a sqrt(T) / phi
+  // derived constants, so that the node code divides by no parameter
+  R inv_m[MMAX];              // 1 / m_a
+  R mum[MMAX];                // mu_ref,a / m_a
+  R Kc;                       // R_U^2 T_ref^1.5 / P_ref: 1/tau_ab = Kc (sum f / phi) sqrt(T) invDmm_ab
   R rho_in[2][MMAX];          // reservoir densities [kg/m^3]
   R T_in[2];
   R kappa_thr;
@@ -93,13 +97,28 @@ template <class R> struct ScalarTraits { static constexpr bool single = sizeof(R
 template <class R> struct MathOps;
 template <> struct MathOps<float> {
   static LBM_HD float sqrt(float v) { return sqrtf(v); }
+  static LBM_HD float rsqrt(float v) {
+#ifdef __CUDA_ARCH__
+    return rsqrtf(v);
+#else
+    return 1.0f / sqrtf(v);
+#endif
+  }
   static LBM_HD float pow(float a, float b) { return powf(a, b); }
 };
 template <> struct MathOps<double> {
   static LBM_HD double sqrt(double v) { return ::sqrt(v); }
+  static LBM_HD double rsqrt(double v) {
+#ifdef __CUDA_ARCH__
+    return ::rsqrt(v);
+#else
+    return 1.0 / ::sqrt(v);
+#endif
+  }
   static LBM_HD double pow(double a, double b) { return ::pow(a, b); }
 };
 template <class R> LBM_HD R sqrt_(R v) { return MathOps<R>::sqrt(v); }
+template <class R> LBM_HD R rsqrt_(R v) { return MathOps<R>::rsqrt(v); }
 template <class R> LBM_HD R pow_(R a, R b) { return MathOps<R>::pow(a, b); }
 template <class R> LBM_HD bool finite_(R v) { return v == v && v - v == v - v; }
 

@@ -112,6 +112,10 @@ struct MathOps<Dual<B, K>> {
     const B s = MathOps<B>::sqrt(x.v);
     return chain(x, s, B(0.5) / s);
   }
+  static LBM_HD Dual<B, K> rsqrt(const Dual<B, K>& x) {
+    const B r = MathOps<B>::rsqrt(x.v);
+    return chain(x, r, B(-0.5) * r * r * r);
+  }
   static LBM_HD Dual<B, K> pow(const Dual<B, K>& x, const Dual<B, K>& e) {
     // exponents are parameters of the transport model: no derivative
     const B p = MathOps<B>::pow(x.v, e.v);

@@ -11,9 +11,14 @@
 // re-reads hit L2) and written once.
 #pragma once
 
-#include "lbm_compact.cuh"
+#include "lbm_twopass.cuh"
 
 namespace lbm {
+
+LBM_HD int modp(int v, int n) {
+  int r = v % n;
+  return r < 0 ? r + n : r;
+}
 
 template <int D, int M, bool EN>
 struct FusedLayout {
@@ -25,11 +30,6 @@ constexpr size_t fused_smem_bytes() {
   return sizeof(R) * 3 * FusedLayout<D, M, EN>::NF * (TX + 2) * ((D == 3) ? TY + 2 : 1);
 }
 
-LBM_HD int modp(int v, int n) {
-  int r = v % n;
-  return r < 0 ? r + n : r;
-}
-
 template <class R, int D, int M, bool EN, int TX, int TY, int SEG>
 __global__ void __launch_bounds__(TX * TY) k_fused(Params<R> p, InletTables<R> it, StepArgs<R> a) {
   constexpr int NT = TX * TY;
@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(TX * TY) k_fused(Params<R> p, InletTables<R> i
   constexpr int PY = (D == 3) ? TY + 2 : 1;
   constexpr int PN = PX * PY;
   constexpr int NF = FusedLayout<D, M, EN>::NF;
+  constexpr int LQ = (M + 1 + (EN ? 1 : 0)) * Lat<D>::Q;
   extern __shared__ unsigned char smem_raw[];
   R* ring = reinterpret_cast<R*>(smem_raw);           // [3][NF][PN]
 
@@ -66,24 +67,14 @@ __global__ void __launch_bounds__(TX * TY) k_fused(Params<R> p, InletTables<R> i
         y = mw;
         z = 0;
       }
-      Site<R, D> st;
-      st.init(p, x, y, z);
-      Ghost<R, D> gh;
-      gh.side = -1;
-      if (st.has_ghost()) ghost_velocity<R, D, M>(p, a.src, a.phi, x, y, z, gh);
+      const int n = x + p.nx * (y + p.ny * z);
+      R P[LQ];
+      pull_node<R, D, M, EN>(p, it, a.src, a.phi, x, y, z, P);
       Moments<R, D, M, EN, false> mo;
-      moments_rt<R, D, M, EN, false>(p, it, a.src, st, gh, mo);
+      moments_gen<R, D, M, EN, false>(ArrayPull<R, D>{P}, mo);
       State<R, D, M> s;
-      s.template from_moments<EN, false>(p, mo, a.phi[st.n], EN ? R(0) : a.Tfix[st.n]);
-#pragma unroll
-      for (int b = 0; b < D; ++b) {
-        dstp[b * PN + e] = s.u[b];
-        dstp[(D + b) * PN + e] = s.Pi(b);
-      }
-      if (EN) {
-#pragma unroll
-        for (int k = 0; k < M; ++k) dstp[(2 * D + k) * PN + e] = s.Y[k];
-      }
+      s.template from_moments<EN, false>(p, mo, a.phi[n], EN ? R(0) : a.Tfix[n]);
+      macro_fields<R, D, M, EN>(s, [&](int k, const R& v) { dstp[k * PN + e] = v; });
     }
   };
   auto slot_of = [](int r) { return (r + 1) % 3; };    // r = m - m0 in [-1, SEG]
@@ -101,15 +92,14 @@ __global__ void __launch_bounds__(TX * TY) k_fused(Params<R> p, InletTables<R> i
     if (active) {
       const int m = m0 + r;
       const int x = xi, y = (D == 3) ? yi : m, z = (D == 3) ? m : 0;
-      Site<R, D> st;
-      st.init(p, x, y, z);
-      Ghost<R, D> gh;
-      gh.side = -1;
-      if (st.has_ghost()) ghost_velocity<R, D, M>(p, a.src, a.phi, x, y, z, gh);
+      const int n = x + p.nx * (y + p.ny * z);
+      R P[LQ];
+      pull_node<R, D, M, EN>(p, it, a.src, a.phi, x, y, z, P);
+      ArrayPull<R, D> pf{P};
       Moments<R, D, M, EN, true> mo;
-      moments_rt<R, D, M, EN, true>(p, it, a.src, st, gh, mo);
+      moments_gen<R, D, M, EN, true>(pf, mo);
       State<R, D, M> s;
-      s.template from_moments<EN, true>(p, mo, a.phi[st.n], EN ? R(0) : a.Tfix[st.n]);
+      s.template from_moments<EN, true>(p, mo, a.phi[n], EN ? R(0) : a.Tfix[n]);
       // gradient inputs from the ring (isotropic stencil, weights 3 w_i)
       Grad<R, D, M, EN> gr;
       gr.divu = R(0);
@@ -119,9 +109,10 @@ __global__ void __launch_bounds__(TX * TY) k_fused(Params<R> p, InletTables<R> i
 #pragma unroll
         for (int k = 0; k < M; ++k) gr.dY[k][b] = R(0);
       }
-      for_each_dir<D>([&](int i, int cx, int cy, int cz) {
-        const int c2 = cx * cx + cy * cy + cz * cz;
-        if (c2 == 0) return;
+      Unroll<0, Lat<D>::Q>::run([&](auto ic) {
+        constexpr int I = decltype(ic)::value;
+        constexpr int cx = c_of<D>(I, 0), cy = c_of<D>(I, 1), cz = c_of<D>(I, 2);
+        if (csq_of<D>(I) == 0) return;
         const R w = R(3) * (cx == 0 ? R(2) / R(3) : R(1) / R(6)) * (cy == 0 ? R(2) / R(3) : R(1) / R(6)) *
                     ((D == 3) ? (cz == 0 ? R(2) / R(3) : R(1) / R(6)) : R(1));
         const int dm = (D == 3) ? cz : cy;                 // march-axis offset
@@ -140,7 +131,7 @@ __global__ void __launch_bounds__(TX * TY) k_fused(Params<R> p, InletTables<R> i
           }
         }
       });
-      collide_rt<R, D, M, EN>(p, it, a.src, st, gh, mo, s, gr, a.dst, a.status);
+      collide_gen<R, D, M, EN>(p, pf, n, mo, s, gr, a.dst, a.status);
     }
     __syncthreads();
   }

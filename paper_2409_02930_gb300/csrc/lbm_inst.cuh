@@ -1,11 +1,10 @@
 // Instantiates the step kernels for one (precision, dimension); the including
 // file defines LBM_REAL, LBM_DIM and LBM_OPS_NAME.
 #include "lbm_fused.cuh"
-#include "lbm_kernels.cuh"
 #include "lbm_march2d.cuh"
 #include "lbm_ops.h"
+#include "lbm_split3d.cuh"
 #include "lbm_staged.cuh"
-#include "lbm_surface.cuh"
 
 namespace lbm {
 namespace {
@@ -27,15 +26,41 @@ int configure(Kern kern, size_t smem, bool& done) {
 template <class R, int D, int M, bool EN>
 struct Launch {
   static int grid(int N) { return (N + 255) / 256; }
+  // 3-D: the step split by lattice, NB = 32 nodes and one warp per lattice in a block
+  static constexpr int NB = 32, L = M + 1 + (EN ? 1 : 0);
+  template <bool AUX>
+  static int macro3(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, R* aux, cudaStream_t s) {
+    if constexpr (D == 3) {
+      constexpr size_t smem = split_smem_bytes<R, M, EN>(NB, false);
+      k_macro3<R, M, EN, NB, AUX><<<(p.N + NB - 1) / NB, NB * L, smem, s>>>(p, it, a, aux);
+    }
+    return 0;
+  }
+  template <bool SRC, int MINB>
+  static int collide3(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, const double* src,
+                      cudaStream_t s) {
+    if constexpr (D == 3) {
+      constexpr size_t smem = split_smem_bytes<R, M, EN>(NB, true);
+      auto kern = k_collide3<R, M, EN, NB, SRC, MINB>;
+      static bool done = false;
+      if (configure(kern, smem, done)) return -1;
+      kern<<<(p.N + NB - 1) / NB, NB * L, smem, s>>>(p, it, a, src);
+    }
+    return 0;
+  }
+  static constexpr int kMinB = sizeof(R) == 4 ? 2 : 1;
   static void macro(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
-    k_macro<R, D, M, EN><<<grid(p.N), 256, 0, s>>>(p, it, a);
+    if constexpr (D == 3) macro3<false>(p, it, a, nullptr, s);
+    else k_macro<R, D, M, EN><<<grid(p.N), 256, 0, s>>>(p, it, a);
   }
   static void collide(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
-    k_collide<R, D, M, EN><<<grid(p.N), 256, 0, s>>>(p, it, a);
+    if constexpr (D == 3) collide3<false, kMinB>(p, it, a, nullptr, s);
+    else k_collide<R, D, M, EN><<<grid(p.N), 256, 0, s>>>(p, it, a);
   }
   // fused step, shared-memory halo ring, tile TX x TY marching SEG planes
   template <int TX, int TY, int SEG>
   static int fused_tile(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
+    static_assert(D == 2, "fused tiles are a 2-D form");
     constexpr size_t smem = fused_smem_bytes<R, D, M, EN, TX, TY>();
     auto kern = k_fused<R, D, M, EN, TX, TY, SEG>;
     static bool done = false;
@@ -108,24 +133,6 @@ struct Launch {
       return 0;
     }
   }
-  // the staged form with the gradient inputs computed once per node in a pass
-  // of their own (3-D; the macro buffer holds them after the macro fields)
-  template <int TB>
-  static int staged_grad(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
-    constexpr size_t smem = sizeof(R) * (size_t)n_pops<R, D, M, EN>() * TB;
-    if constexpr (D != 3 || smem > kMaxSmem) {
-      return -1;
-    } else {
-      auto kern = k_collide_staged_g<R, D, M, EN, TB>;
-      auto kmac = k_macro_staged<R, D, M, EN, TB>;
-      static bool done = false, done_mac = false;
-      if (configure(kern, smem, done) || configure(kmac, smem, done_mac)) return -1;
-      kmac<<<(p.N + TB - 1) / TB, TB, smem, s>>>(p, it, a);
-      k_grad<R, D, M, EN><<<(p.N + 255) / 256, 256, 0, s>>>(p, a);
-      kern<<<(p.N + TB - 1) / TB, TB, smem, s>>>(p, it, a);
-      return 0;
-    }
-  }
   static int fused(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, int v, cudaStream_t s) {
     if constexpr (D == 2) {
       switch (v) {
@@ -142,13 +149,14 @@ struct Launch {
         default: return -1;
       }
     } else {
+      macro3<false>(p, it, a, nullptr, s);
       switch (v) {
-        case 0: return fused_tile<32, 4, 16>(p, it, a, s);
-        case 1: return fused_tile<32, 8, 16>(p, it, a, s);
-        case 2: return fused_tile<32, 4, 8>(p, it, a, s);
-        case 3: return staged<64>(p, it, a, s);
-        case 4: return staged<32>(p, it, a, s);
-        case 5: return staged_grad<64>(p, it, a, s);
+        case 0: return collide3<false, 1>(p, it, a, nullptr, s);
+        case 1: return collide3<false, 2>(p, it, a, nullptr, s);
+        case 2: return collide3<false, sizeof(R) == 4 ? 3 : 1>(p, it, a, nullptr, s);
+        case 3: return collide3<false, sizeof(R) == 4 ? 4 : 1>(p, it, a, nullptr, s);
+        case 4: return collide3<false, kMinB>(p, it, a, nullptr, s);
+        case 5: return collide3<false, kMinB>(p, it, a, nullptr, s);
         default: return -1;
       }
     }
@@ -165,22 +173,15 @@ struct Launch {
   static constexpr bool has_react = (D == 3 && M == 6 && EN);
   static void react_macro(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, const ReactArgs& ra,
                           cudaStream_t s) {
-    if constexpr (has_react) k_macro_react<R, D, M, EN><<<(p.N + 127) / 128, 128, 0, s>>>(p, it, a, ra);
+    if constexpr (has_react) {
+      R* aux = a.mac + (size_t)(2 * D + M) * p.N;
+      macro3<true>(p, it, a, aux, s);
+      k_source<R, M><<<(p.N + 127) / 128, 128, 0, s>>>(p.N, aux, a.phi, a.status, ra);
+    }
   }
   static void react_collide(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, const ReactArgs& ra,
                             cudaStream_t s) {
-    if constexpr (has_react) {
-      // node populations staged in shared memory (TB x 216 values per block)
-      constexpr int TB = sizeof(R) == 4 ? 64 : 32;
-      constexpr size_t smem = sizeof(R) * (size_t)n_pops<R, D, M, EN>() * TB;
-      auto kern = k_collide_react_staged<R, D, M, EN, TB>;
-      static bool done = false;
-      if (configure(kern, smem, done)) {
-        k_collide_react<R, D, M, EN><<<(p.N + 127) / 128, 128, 0, s>>>(p, it, a, ra);
-        return;
-      }
-      kern<<<(p.N + TB - 1) / TB, TB, smem, s>>>(p, it, a, ra);
-    }
+    if constexpr (has_react) collide3<true, kMinB>(p, it, a, ra.src, s);
   }
   static Ops<R> ops() {
     return Ops<R>{macro, collide, fused, n_variants, init, moments, has_react ? react_macro : nullptr,

@@ -16,7 +16,7 @@
 // missing populations are reservoir equilibria computed on the fly).
 #pragma once
 
-#include "lbm_compact.cuh"
+#include "lbm_twopass.cuh"
 #include "lbm_tma.cuh"
 
 namespace lbm {
@@ -37,9 +37,7 @@ template <class R, int D>
 struct SmemPull {
   const R* col;
   int stride;
-  static constexpr bool kUnroll = (D == 2);
-  LBM_HD int prep(int, int, int) const { return 0; }
-  LBM_HD R get(int, int l, int i, int, int, int) const { return col[(l * Lat<D>::Q + i) * stride]; }
+  LBM_HD R get(int l, int i) const { return col[(l * Lat<D>::Q + i) * stride]; }
 };
 
 // Row-box layout of the TMA form: for each row buffer, one chunk per
@@ -70,9 +68,7 @@ struct RowBoxLayout {
 template <class R, int CH, int LW>
 struct RowPull {
   const R* col;                      // chunk base + t + c0
-  static constexpr bool kUnroll = true;
-  LBM_HD int prep(int, int, int) const { return 0; }
-  LBM_HD R get(int, int l, int i, int cx, int, int) const { return col[i * CH + l * LW - cx]; }
+  LBM_HD R get(int l, int i) const { return col[i * CH + l * LW - (i % 3 - 1)]; }
 };
 
 // PD rows are prefetched ahead; PD + 2 row buffers are in use at a time
@@ -229,11 +225,9 @@ __global__ void __launch_bounds__(TX, MINB)
       const int n = xm + p.nx * y;
       Moments<R, D, M, EN, false> mo;
       if (slow) {
-        Site<R, D> st;
-        st.init(p, xm, y, 0);
-        Ghost<R, D> gh;
-        ghost_velocity<R, D, M>(p, a.src, a.phi, xm, y, 0, gh);
-        moments_rt<R, D, M, EN, false>(p, it, a.src, st, gh, mo);
+        R Pn[NL * Q];
+        pull_node<R, D, M, EN>(p, it, a.src, a.phi, xm, y, 0, Pn);
+        moments_gen<R, D, M, EN, false>(ArrayPull<R, D>{Pn}, mo);
       } else if constexpr (TMA) {
         RowPull<R, LB::CH, LB::W> pf{col_of(buf_of(s))};
         moments_gen<R, D, M, EN, false>(pf, mo);
@@ -245,15 +239,7 @@ __global__ void __launch_bounds__(TX, MINB)
       State<R, D, M> st;
       st.template from_moments<EN, false>(p, mo, slow ? a.phi[n] : sf[0], EN ? R(0) : (slow ? a.Tfix[n] : sf[SSTR]));
       R* rs = ring + (size_t)slot_of(s) * NF * TX + t;
-#pragma unroll
-      for (int b = 0; b < D; ++b) {
-        rs[b * TX] = st.u[b];
-        rs[(D + b) * TX] = st.Pi(b);
-      }
-      if (EN) {
-#pragma unroll
-        for (int k = 0; k < M; ++k) rs[(2 * D + k) * TX] = st.Y[k];
-      }
+      macro_fields<R, D, M, EN>(st, [&](int k, const R& v) { rs[k * TX] = v; });
       if (KEEP) st_new = st;
     }
     if (s + PD <= mend) {
@@ -276,13 +262,12 @@ __global__ void __launch_bounds__(TX, MINB)
       const int y = s - 1;
       const int n = xt + p.nx * y;
       Moments<R, D, M, EN, true> mo;
-      Site<R, D> site;
-      site.init(p, xt, y, 0);
-      Ghost<R, D> gh;
-      gh.side = -1;
+      R Pn[INLET ? NL * Q : 1];
       if (slow) {
-        ghost_velocity<R, D, M>(p, a.src, a.phi, xt, y, 0, gh);
-        moments_rt<R, D, M, EN, true>(p, it, a.src, site, gh, mo);
+        if constexpr (INLET) {
+          pull_node<R, D, M, EN>(p, it, a.src, a.phi, xt, y, 0, Pn);
+          moments_gen<R, D, M, EN, true>(ArrayPull<R, D>{Pn}, mo);
+        }
       } else if constexpr (TMA) {
         RowPull<R, LB::CH, LB::W> pf{col_of(buf_of(y))};
         moments_gen<R, D, M, EN, true>(pf, mo);
@@ -331,8 +316,7 @@ __global__ void __launch_bounds__(TX, MINB)
         }
       }
       if (slow) {
-        GlobalPull<R, D, M, EN> pf{p, it, a.src, site, gh};
-        collide_gen<R, D, M, EN>(p, pf, n, mo, st, gr, a.dst, a.status);
+        if constexpr (INLET) collide_gen<R, D, M, EN>(p, ArrayPull<R, D>{Pn}, n, mo, st, gr, a.dst, a.status);
       } else if constexpr (TMA) {
         RowPull<R, LB::CH, LB::W> pf{col_of(buf_of(y))};
         collide_gen<R, D, M, EN>(p, pf, n, mo, st, gr, a.dst, a.status);

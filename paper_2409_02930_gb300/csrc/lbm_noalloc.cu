@@ -23,7 +23,7 @@
 #include <mutex>
 
 #include "../../include/lbm.h"
-#include "lbm_kernels.cuh"
+#include "lbm_twopass.cuh"
 
 namespace lbm {
 void make_params(const lbm_config* c, Params<double>& p, InletTables<double>& it, double& dt, double& cvel);
@@ -64,10 +64,11 @@ void to_precision(const lbm::Params<double>& d, lbm::Params<R>& r, const lbm::In
                   lbm::InletTables<R>& ri) {
   r.nx = d.nx; r.ny = d.ny; r.nz = d.nz; r.N = d.N;
   r.bc_lo = d.bc_lo; r.bc_hi = d.bc_hi; r.knudsen = d.knudsen;
-  r.RU = (R)d.RU;
+  r.RU = (R)d.RU; r.Kc = (R)d.Kc;
   for (int a = 0; a < lbm::MMAX; ++a) {
     r.m[a] = (R)d.m[a]; r.Ra[a] = (R)d.Ra[a]; r.muref[a] = (R)d.muref[a];
     r.cvR[a] = (R)d.cvR[a]; r.U0[a] = (R)d.U0[a]; r.knc[a] = (R)d.knc[a];
+    r.inv_m[a] = (R)d.inv_m[a]; r.mum[a] = (R)d.mum[a];
     for (int b = 0; b < lbm::MMAX; ++b) r.invDmm[a][b] = (R)d.invDmm[a][b];
     r.rho_in[0][a] = (R)d.rho_in[0][a]; r.rho_in[1][a] = (R)d.rho_in[1][a];
   }

@@ -16,7 +16,7 @@
 // and loses the electric power of the current (Sec. 4.2).
 #pragma once
 
-#include "lbm_compact.cuh"
+#include "lbm_twopass.cuh"
 
 namespace lbm {
 
@@ -244,61 +244,24 @@ struct ReactArgs {
   double* src;             // [M + 2][N]: rhodot_a, then dU, then the volumetric current
 };
 
-// Pass 1: macro fields (as k_macro) plus the surface source of the node.
-template <class R, int D, int M, bool EN>
-__global__ void __launch_bounds__(128) k_macro_react(Params<R> p, InletTables<R> it, StepArgs<R> a, ReactArgs ra) {
+// Surface source of every node, from the species sums and temperatures that
+// the macro-field pass left in aux ([M + 1][N]).
+template <class R, int M>
+__global__ void __launch_bounds__(128) k_source(int N, const R* __restrict__ aux, const R* __restrict__ phi,
+                                                int* status, ReactArgs ra) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= p.N) return;
-  macro_node<R, D, M, EN>(p, it, a, n);
-  // the surface source needs the streamed species densities and temperature
-  int x, y, z;
-  node_xyz<R, D>(p, n, x, y, z);
-  Site<R, D> st;
-  st.init(p, x, y, z);
-  Ghost<R, D> gh;
-  gh.side = -1;
-  if (st.has_ghost()) ghost_velocity<R, D, M>(p, a.src, a.phi, x, y, z, gh);
-  Moments<R, D, M, EN, false> mo;
-  moments_rt<R, D, M, EN, false>(p, it, a.src, st, gh, mo);
-  State<R, D, M> s;
-  s.template from_moments<EN, false>(p, mo, a.phi[n], EN ? R(0) : a.Tfix[n]);
+  if (n >= N) return;
   const MechDev& mc = *ra.mech;
   double rho[MMAX], Xs0[SMAX], Xs1[SMAX], rd[MMAX], dU = 0.0, cur = 0.0;
-  for (int k = 0; k < M; ++k) rho[k] = (double)s.rho_a[k];
-  for (int k = 0; k < mc.S; ++k) Xs0[k] = ra.Xs_in[(size_t)k * p.N + n];
+  const R ph = phi[n];
+  for (int k = 0; k < M; ++k) rho[k] = (double)(aux[(size_t)k * N + n] / ph);
+  for (int k = 0; k < mc.S; ++k) Xs0[k] = ra.Xs_in[(size_t)k * N + n];
   const double dphi_n = mc.dphi_field ? mc.dphi_field[n] : mc.dphi;
-  surface_source_dev<M, R>(mc, (double)s.T, rho, (double)s.phi, Xs0, rd, Xs1, dU, cur, dphi_n, a.status);
-  for (int k = 0; k < M; ++k) ra.src[(size_t)k * p.N + n] = rd[k];
-  ra.src[(size_t)M * p.N + n] = dU;
-  ra.src[(size_t)(M + 1) * p.N + n] = cur;
-  for (int k = 0; k < mc.S; ++k) ra.Xs_out[(size_t)k * p.N + n] = Xs1[k];
-}
-
-// Pass 2: node update with the reaction sources.
-template <class R, int D, int M, bool EN>
-__global__ void __launch_bounds__(128) k_collide_react(Params<R> p, InletTables<R> it, StepArgs<R> a, ReactArgs ra) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= p.N) return;
-  int x, y, z;
-  node_xyz<R, D>(p, n, x, y, z);
-  Site<R, D> st;
-  st.init(p, x, y, z);
-  Ghost<R, D> gh;
-  gh.side = -1;
-  if (st.has_ghost()) ghost_velocity<R, D, M>(p, a.src, a.phi, x, y, z, gh);
-  Moments<R, D, M, EN, true> mo;
-  moments_rt<R, D, M, EN, true>(p, it, a.src, st, gh, mo);
-  State<R, D, M> s;
-  s.template from_moments<EN, true>(p, mo, a.phi[n], EN ? R(0) : a.Tfix[n]);
-  Grad<R, D, M, EN> gr;
-  const R* __restrict__ mac = a.mac;
-  const int N = p.N;
-  gr.compute(p, x, y, z, [&](int k, int nb) { return mac[(size_t)k * N + nb]; });
-  NodeSource<R> src;
-  for (int k = 0; k < M; ++k) src.rhodot[k] = (R)ra.src[(size_t)k * N + n];
-  src.dU = (R)ra.src[(size_t)M * N + n];
-  GlobalPull<R, D, M, EN> pf{p, it, a.src, st, gh};
-  collide_gen<R, D, M, EN, GlobalPull<R, D, M, EN>, true>(p, pf, n, mo, s, gr, a.dst, a.status, &src);
+  surface_source_dev<M, R>(mc, (double)aux[(size_t)M * N + n], rho, (double)ph, Xs0, rd, Xs1, dU, cur, dphi_n, status);
+  for (int k = 0; k < M; ++k) ra.src[(size_t)k * N + n] = rd[k];
+  ra.src[(size_t)M * N + n] = dU;
+  ra.src[(size_t)(M + 1) * N + n] = cur;
+  for (int k = 0; k < mc.S; ++k) ra.Xs_out[(size_t)k * N + n] = Xs1[k];
 }
 
 }  // namespace lbm
