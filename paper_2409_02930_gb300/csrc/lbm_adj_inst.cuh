@@ -5,13 +5,6 @@
 namespace lbm {
 namespace {
 
-// dual lanes of the node-update evaluations: fewer lanes spill less (with
-// populations seeded, FP32 took 1.65 ms per adjoint step of the 256x256 slab
-// with 2 lanes and 2.87 ms with 4); with the moments seeded, 4 lanes in FP64
-// push the node code past the register file into a 13 KB stack frame
-template <class B> constexpr int kLanesOf() { return 2; }
-constexpr int kLanesSmall = 8;   // dual lanes of the macro-field and reservoir-ghost evaluations
-
 template <class To, class From>
 void params_cast(const Params<From>& s, Params<To>& d) {
   d.nx = s.nx; d.ny = s.ny; d.nz = s.nz; d.N = s.N;
@@ -32,31 +25,26 @@ void params_cast(const Params<From>& s, Params<To>& d) {
 
 template <class B, int D, int M, bool EN>
 struct AdjLaunch {
-  static constexpr int K = kLanesOf<B>(), KS = kLanesSmall;
-  template <int KK>
-  static AdjParams<B, KK> make(const Params<B>& p) {
-    AdjParams<B, KK> ap;
-    params_cast(p, ap.pz);
-    ap.pz.N = 1;                 // node-local evaluation into a local array
-    ap.pk = ap.pz;
-    for (int a = 0; a < MMAX; ++a) ap.pk.knc[a].d[0] = p.knc[a];
-    return ap;
-  }
   static int grid(int n, int b) { return (n + b - 1) / b; }
-  static int collide(const Params<B>& p, const InletTables<B>& it, const AdjArgs<B>& a, cudaStream_t s) {
-    k_adj_collide<B, D, M, EN, K><<<grid(p.N, 128), 128, 0, s>>>(p, it, a, make<K>(p));
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+  static int done() { return cudaGetLastError() == cudaSuccess ? 0 : -1; }
+  static int fields(const Params<B>& p, const InletTables<B>& it, const AdjArgs<B>& a, cudaStream_t s) {
+    k_adj_fields<B, M, EN><<<grid(p.N, 128), 128, 0, s>>>(p, it, a);
+    return done();
   }
-  static int macro(const Params<B>& p, const InletTables<B>& it, const AdjArgs<B>& a, cudaStream_t s) {
-    k_adj_macro<B, D, M, EN, KS><<<grid(p.N, 128), 128, 0, s>>>(p, it, a, make<KS>(p));
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+  static int collide(const Params<B>& p, const InletTables<B>& it, const AdjArgs<B>& a, cudaStream_t s) {
+    k_adj_collide<B, M, EN><<<grid(p.N, 64), 64, 0, s>>>(p, it, a);
+    return done();
+  }
+  static int macro(const Params<B>& p, const AdjArgs<B>& a, bool seed, cudaStream_t s) {
+    if (seed) k_adj_macro<B, M, EN, false><<<grid(p.N, 128), 128, 0, s>>>(p, a);
+    else k_adj_macro<B, M, EN, true><<<grid(p.N, 128), 128, 0, s>>>(p, a);
+    return done();
   }
   static int ghost(const Params<B>& p, const InletTables<B>& it, const AdjArgs<B>& a, cudaStream_t s) {
-    k_adj_ghost<B, D, M, EN, KS><<<grid(p.ny * p.nz, 128), 128, 0, s>>>(p, it, a, make<KS>(p));
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
-  }
-  static void stream(const Params<B>& p, const AdjArgs<B>& a, cudaStream_t s) {
-    k_adj_stream<B, D, M, EN><<<grid(p.N, 256), 256, 0, s>>>(p, a);
+    Params<Dual<B, 3>> pd;
+    params_cast(p, pd);
+    k_adj_ghost<B, M, EN><<<dim3(grid(p.ny, 32), p.nx > 3 ? 2 : 1), 32, 0, s>>>(p, it, a, pd);
+    return done();
   }
   static void seed_flux(const Params<B>& p, const AdjArgs<B>& a, int species, int axis, int xo, double w,
                         cudaStream_t s) {
@@ -66,7 +54,7 @@ struct AdjLaunch {
                    double cvel, double RU, const AdjArgs<B>& a, cudaStream_t s) {
     k_adj_init<B, D, M, EN><<<grid(p.N, 128), 128, 0, s>>>(p, X, T, P, U, cvel, RU, a);
   }
-  static AdjOps<B> ops() { return AdjOps<B>{collide, macro, ghost, stream, seed_flux, init, n_grad<D, M, EN>()}; }
+  static AdjOps<B> ops() { return AdjOps<B>{fields, collide, macro, ghost, seed_flux, init, n_grad<D, M, EN>(), n_sums<M>()}; }
 };
 
 }  // namespace

@@ -44,7 +44,7 @@ int run_adjoint(lbm_ctx* x, const lbm::Ops<B>& ops, const lbm::Params<B>& p, con
   const int nck = n_steps > 0 ? (n_steps + C - 1) / C : 0;
   cudaStream_t s = x->stream;
   Scratch sc;
-  B *ck = nullptr, *seg = nullptr, *lamA = nullptr, *lamB = nullptr, *Pbar = nullptr, *Gbar = nullptr;
+  B *ck = nullptr, *seg = nullptr, *lamA = nullptr, *lamB = nullptr, *Pbar = nullptr, *Gbar = nullptr, *sums = nullptr;
   double *phibar = nullptr, *kbar = nullptr, *jbuf = nullptr;
   cudaError_t e = sc.alloc(&ck, state * (nck > 0 ? nck : 1));
   if (e == cudaSuccess) e = sc.alloc(&seg, state * (C > 1 ? C - 1 : 1));
@@ -52,6 +52,7 @@ int run_adjoint(lbm_ctx* x, const lbm::Ops<B>& ops, const lbm::Params<B>& p, con
   if (e == cudaSuccess) e = sc.alloc(&lamB, state);
   if (e == cudaSuccess) e = sc.alloc(&Pbar, state);
   if (e == cudaSuccess) e = sc.alloc(&Gbar, (size_t)adj.n_grad * N * sizeof(B));
+  if (e == cudaSuccess) e = sc.alloc(&sums, (size_t)adj.n_sums * N * sizeof(B));
   if (e == cudaSuccess) e = sc.alloc(&phibar, N * sizeof(double));
   if (e == cudaSuccess) e = sc.alloc(&kbar, N * sizeof(double));
   if (e == cudaSuccess) e = sc.alloc(&jbuf, (size_t)x->M * x->D * N * sizeof(double));
@@ -99,11 +100,11 @@ int run_adjoint(lbm_ctx* x, const lbm::Ops<B>& ops, const lbm::Params<B>& p, con
   // ---- adjoint of the final state ---------------------------------------------
   cudaMemsetAsync(phibar, 0, N * sizeof(double), s);
   cudaMemsetAsync(kbar, 0, N * sizeof(double), s);
-  lbm::AdjArgs<B> a{cur, mac, phi, Tfix, nullptr, Pbar, Gbar, phibar, kbar, lamA, x->status};
+  lbm::AdjArgs<B> a{cur, mac, sums, phi, Tfix, nullptr, Pbar, Gbar, phibar, kbar, lamA, x->status};
   adj.seed_flux(p, a, obj->species, obj->axis, obj->plane, obj->weight, s);
   const bool inlet = (p.bc_lo == lbm::BC_INLET) || (p.bc_hi == lbm::BC_INLET);
-  if (inlet && adj.ghost(p, it, a, s)) return adj_fail(x, LBM_ERR_CUDA, "adjoint ghost launch");
-  adj.stream(p, a, s);
+  if (adj.macro(p, a, true, s) || (inlet && adj.ghost(p, it, a, s)))
+    return adj_fail(x, LBM_ERR_CUDA, "adjoint seed launch");
   B* lam1 = lamA;     // adjoint of f^{k+1}
   B* lam0 = lamB;
   // ---- reverse sweep, one checkpoint segment at a time ---------------------
@@ -114,12 +115,10 @@ int run_adjoint(lbm_ctx* x, const lbm::Ops<B>& ops, const lbm::Params<B>& p, con
     for (int k = k0; k + 1 < k1; ++k) step(state_of(k), seg + (size_t)(k - k0) * LQN);
     for (int k = k1 - 1; k >= k0; --k) {
       const B* f = state_of(k);
-      lbm::StepArgs<B> sa{f, nullptr, phi, Tfix, mac, x->status};
-      ops.macro(p, it, sa, s);
-      lbm::AdjArgs<B> aa{f, mac, phi, Tfix, lam1, Pbar, Gbar, phibar, kbar, lam0, x->status};
-      if (adj.collide(p, it, aa, s) || adj.macro(p, it, aa, s) || (inlet && adj.ghost(p, it, aa, s)))
+      lbm::AdjArgs<B> aa{f, mac, sums, phi, Tfix, lam1, Pbar, Gbar, phibar, kbar, lam0, x->status};
+      if (adj.fields(p, it, aa, s) || adj.collide(p, it, aa, s) || adj.macro(p, aa, false, s) ||
+          (inlet && adj.ghost(p, it, aa, s)))
         return adj_fail(x, LBM_ERR_CUDA, "adjoint kernel launch");
-      adj.stream(p, aa, s);
       B* t = lam1;
       lam1 = lam0;
       lam0 = t;
@@ -127,7 +126,7 @@ int run_adjoint(lbm_ctx* x, const lbm::Ops<B>& ops, const lbm::Params<B>& p, con
   }
   // ---- initial equilibria ------------------------------------------------------
   {
-    lbm::AdjArgs<B> aa{nullptr, mac, phi, Tfix, nullptr, Pbar, Gbar, phibar, kbar, lam1, x->status};
+    lbm::AdjArgs<B> aa{nullptr, mac, sums, phi, Tfix, nullptr, Pbar, Gbar, phibar, kbar, lam1, x->status};
     adj.init(p, x->init_X, x->init_T, x->init_P, x->init_U, x->cvel, R_UNIV_SI_ADJ, aa, s);
   }
   e = cudaGetLastError();
