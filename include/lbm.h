@@ -160,14 +160,13 @@ int lbm_create(lbm_ctx** out, const lbm_config* cfg);
  * lbm_create would (each case gets its own lattice scaling from its dx,
  * theta_max and T_scale); every case must have nz = 1, no surface mechanism
  * and the same M, energy flag and precision, with (M, energy) = (2, off) or
- * (3, on); the stream of cfgs[0] is used.  The cases are stepped together:
- * each lbm_step launches two persistent kernels (macro-field pass, node
- * update) over one work list of node tiles of all cases, replayed from a
- * CUDA graph of 50 steps.  Variants 0..11 select the tile length (64, 128,
- * 256 nodes for (v % 6)/2 = 0, 1, 2), the grid (v even: one block per
- * resident slot of every SM, looping over a contiguous range of tiles; v odd:
- * one block per tile) and, for v >= 6, the staging of every node's pulled
- * populations in shared memory; lbm_autotune picks among them.  Per-node outputs
+ * (3, on); the stream of cfgs[0] is used.  The cases are stepped together over
+ * one work list of all cases, replayed from a CUDA graph of 50 steps.
+ * Variants 0..5 launch two kernels per step (macro-field pass, node update)
+ * over runs of 64, 128 or 256 nodes (v / 2), variants 6..11 one kernel over
+ * tiles of 8 x 4, 16 x 4 or 32 x 4 nodes ((v - 6) / 2); v even: one block per
+ * resident slot of every SM, looping over a contiguous range of the list, v
+ * odd: one block per entry.  lbm_autotune picks among them.  Per-node outputs
  * (lbm_moments, populations) are the concatenation over cases, in case
  * order, of each case's single-lattice layout.  Errors as lbm_create, plus
  * LBM_ERR_ARG for n_cases < 1 or cases of different kinds.
@@ -323,15 +322,18 @@ int lbm_get_timing(lbm_ctx* ctx, double* ms_by_kind /* [3] */, long long* launch
  * asynchronous copies, 5 a fused halo tile, 6-7 the staged two-pass form,
  * 8-9 the row march staged by bulk tensor copies (TMA; on lattices whose
  * rows are not a multiple of 16 bytes they run the per-thread-copy march of
- * the same tile shape, variants 2 and 0).
+ * the same tile shape, variants 2 and 0), 10-12 the single-launch form on
+ * tiles of 8 x 4, 16 x 8 and 32 x 4 nodes with the populations in registers.
  * D3Q27: every form is the two-pass step split by lattice (one warp per
  * lattice of 32 nodes); the indices select the registers a thread may use
  * (0: one resident block per SM, 1: two, 2: three, 3: four; 4 and 5 the
  * default).  Every form
  * computes the same step (the gradient stencil is summed in different
  * orders, so the forms agree to rounding).  New contexts use variant 5 in
- * 3-D and, in 2-D, variant 8 on lattices of at least 2^18 nodes without a
- * reservoir face, else the two-pass form; batches use variant 2.  The adjoint's
+ * 3-D and, in 2-D, variant 8 on FP32 lattices of at least 2^18 nodes with nx a
+ * multiple of 4 and no reservoir face, else tiles (10 below 8192 nodes, above
+ * that 12 in FP32 and 11 in FP64; lattices of one or two rows with 8192 nodes
+ * or more: the two-pass form); batches use variant 10.  The adjoint's
  * forward and recompute steps use the context's form.  lbm_autotune times
  * every form for `steps` steps on the
  * current state, restores the state, selects the fastest form and writes its

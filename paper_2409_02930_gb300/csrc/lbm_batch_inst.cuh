@@ -7,59 +7,47 @@ namespace {
 
 template <class R, int D, int M, bool EN>
 struct BatchLaunch {
-  // variant v: tile length kTiles[(v % 6) / 2]; grid mode v % 2; v >= 6 stages populations in shared memory
-  static constexpr int kTiles[3] = {64, 128, 256};
-  static int tile(int v) { return kTiles[(v % 6) / 2]; }
+  // variant v < 6: two passes over runs of 64, 128 or 256 nodes (v / 2); v >= 6:
+  // one pass over tiles of 8 x 4, 16 x 4 or 32 x 4 nodes; v % 2: grid mode
+  static constexpr int kRuns[3] = {64, 128, 256}, kTileX[3] = {8, 16, 32};
+  static void tile(int v, int* tx, int* ty) {
+    *tx = v < 6 ? kRuns[v / 2] : kTileX[(v - 6) / 2];
+    *ty = v < 6 ? 0 : 4;
+  }
+  template <class Kern>
+  static int blocks(Kern kern, int threads) {
+    int n = 0;
+    return (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, 0) == cudaSuccess && n > 0) ? n : 1;
+  }
   template <int TB>
-  static constexpr size_t smem() { return sizeof(R) * (size_t)n_pops<R, D, M, EN>() * TB; }
-  template <int TB>
-  static int occ(bool staged) {
-    int a = 0, b = 0;
-    cudaError_t e1, e2;
-    if (staged) {
-      e1 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_batch_staged<R, D, M, EN, TB, false>, TB, smem<TB>());
-      e2 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch_staged<R, D, M, EN, TB, true>, TB, smem<TB>());
-    } else {
-      e1 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_batch<R, D, M, EN, TB, false>, TB, 0);
-      e2 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_batch<R, D, M, EN, TB, true>, TB, 0);
-    }
-    if (e1 != cudaSuccess) a = 1;
-    if (e2 != cudaSuccess) b = 1;
-    return a < b ? (a > 0 ? a : 1) : (b > 0 ? b : 1);
+  static int runs_occ() {
+    const int a = blocks(k_batch<R, D, M, EN, TB, false>, TB), b = blocks(k_batch<R, D, M, EN, TB, true>, TB);
+    return a < b ? a : b;
   }
   static int occupancy(int v) {
-    const bool staged = v >= 6;
-    switch ((v % 6) / 2) {
-      case 0: return occ<64>(staged);
-      case 1: return occ<128>(staged);
-      default: return occ<256>(staged);
+    switch (v / 2) {
+      case 0: return runs_occ<64>();
+      case 1: return runs_occ<128>();
+      case 2: return runs_occ<256>();
+      case 3: return blocks(k_batch_tile<R, M, EN, 8, 4>, 32);
+      case 4: return blocks(k_batch_tile<R, M, EN, 16, 4>, 64);
+      default: return blocks(k_batch_tile<R, M, EN, 32, 4>, 128);
     }
   }
   template <int TB>
-  static void run(const BatchArgs<R>& b, int grid, int collide, bool staged, cudaStream_t s) {
-    if (staged) {
-      constexpr size_t sm = smem<TB>();
-      if (sm > 48 * 1024) {
-        static bool done = false;
-        if (!done) {
-          cudaFuncSetAttribute(k_batch_staged<R, D, M, EN, TB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-          cudaFuncSetAttribute(k_batch_staged<R, D, M, EN, TB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-          done = true;
-        }
-      }
-      if (collide) k_batch_staged<R, D, M, EN, TB, true><<<grid, TB, sm, s>>>(b);
-      else k_batch_staged<R, D, M, EN, TB, false><<<grid, TB, sm, s>>>(b);
-    } else {
-      if (collide) k_batch<R, D, M, EN, TB, true><<<grid, TB, 0, s>>>(b);
-      else k_batch<R, D, M, EN, TB, false><<<grid, TB, 0, s>>>(b);
-    }
+  static void runs(const BatchArgs<R>& b, int grid, int collide, cudaStream_t s) {
+    if (collide) k_batch<R, D, M, EN, TB, true><<<grid, TB, 0, s>>>(b);
+    else k_batch<R, D, M, EN, TB, false><<<grid, TB, 0, s>>>(b);
   }
   static void pass(const BatchArgs<R>& b, int v, int grid, int collide, cudaStream_t s) {
-    const bool staged = v >= 6;
-    switch ((v % 6) / 2) {
-      case 0: run<64>(b, grid, collide, staged, s); break;
-      case 1: run<128>(b, grid, collide, staged, s); break;
-      default: run<256>(b, grid, collide, staged, s); break;
+    if (v >= 6 && !collide) return;                   // one pass: nothing before the node update
+    switch (v / 2) {
+      case 0: runs<64>(b, grid, collide, s); break;
+      case 1: runs<128>(b, grid, collide, s); break;
+      case 2: runs<256>(b, grid, collide, s); break;
+      case 3: k_batch_tile<R, M, EN, 8, 4><<<grid, 32, 0, s>>>(b); break;
+      case 4: k_batch_tile<R, M, EN, 16, 4><<<grid, 64, 0, s>>>(b); break;
+      default: k_batch_tile<R, M, EN, 32, 4><<<grid, 128, 0, s>>>(b); break;
     }
   }
   static BatchOps<R> ops() { return BatchOps<R>{tile, occupancy, pass, 12}; }

@@ -70,6 +70,27 @@ void convert_inlet(const lbm::InletTables<double>& d, lbm::InletTables<R>& r) {
 // arrays (porosity, X_init, T_init, P_init) that lbm_create reads.
 constexpr int kDefaultWaitLimit = 1 << 22;
 
+// Kernel form of a new single lattice.  3-D: the split step.  2-D, measured in
+// us per step (tiles / row march / two-pass):
+//   FP32 64x40 5.0 / 21.8 / 8.3, 256x256 with reservoirs 14.4 / 73 / 18.5,
+//   512x512 30.8 / 30.9 / 43.7, 701x523 with walls 45 / 58 / 70,
+//   2048x2048 393 / 382 / 697; FP64 512x512 549 / 689 / 608, 256x4 33 / 226 / 60.
+// The row march (bulk tensor copies, rows of whole 16-byte units, no
+// reservoir) is taken from 2^18 FP32 nodes, where its prefetched rows read
+// HBM without stalls; everything else runs on tiles: 8 x 4 below 8192 nodes
+// (one warp each, so that the lattice spreads over the SMs), above that 32 x 4
+// in FP32 (whole lines) and 16 x 8 in FP64 (bound by operations, so the
+// smaller halo counts).  Lattices of one or two rows would leave most of a
+// tile idle and take the two-pass form once they fill the GPU.
+int default_variant(const lbm_config* c) {
+  if (c->nz > 1) return 5;
+  const long long N = (long long)c->nx * c->ny;
+  const bool reservoir = c->bc_lo == LBM_BC_INLET || c->bc_hi == LBM_BC_INLET;
+  if (c->precision == LBM_FP32 && !reservoir && N >= (1 << 18) && c->nx % 4 == 0) return 8;
+  if (c->ny > 4 * 65535 || (c->ny < 3 && N >= 8192)) return -1;
+  return N < 8192 ? 10 : (c->precision == LBM_FP32 ? 12 : 11);
+}
+
 int validate(const lbm_config* c, bool fields = true) {
   if (!c) return fail(nullptr, LBM_ERR_ARG, "null config");
   if (c->nx < 1 || c->ny < 1 || c->nz < 1) return fail(nullptr, LBM_ERR_ARG, "lattice dimensions must be >= 1");
@@ -295,12 +316,7 @@ int lbm_create(lbm_ctx** out, const lbm_config* c) {
   x->S = c->S;
   x->stream = (cudaStream_t)c->stream;
   x->cur = 0;
-  // default form: in 3-D the staged form with a gradient pass; in 2-D the TMA row march
-  // where it fills the GPU (one 32-column block per 8 rows: 1152 blocks at
-  // 512 x 512) and no x face is a reservoir (reservoir columns take a
-  // global-memory path that sets the march's pace), else the two-pass form
-  const bool reservoir = c->bc_lo == LBM_BC_INLET || c->bc_hi == LBM_BC_INLET;
-  x->variant = c->nz > 1 ? 5 : ((!reservoir && x->N >= (1 << 18)) ? 8 : -1);
+  x->variant = default_variant(c);
 
   bool ok = (x->precision == LBM_FP64)
                 ? (x->D == 2 ? lbm::get_ops_f64_2d(x->M, x->energy, &x->od) : lbm::get_ops_f64_3d(x->M, x->energy, &x->od))
@@ -436,7 +452,7 @@ int lbm_create_batch(lbm_ctx** out, int n_cases, const lbm_config* cfgs) {
   x->precision = c0.precision;
   x->stream = (cudaStream_t)c0.stream;
   x->n_cases = n_cases;
-  x->variant = 2;
+  x->variant = 10;                      // one pass over 32 x 4 tiles, resident blocks looping over them
   bool ok = (x->precision == LBM_FP64)
                 ? lbm::get_ops_f64_2d(x->M, x->energy, &x->od) && lbm::get_batch_ops_f64(x->M, x->energy, &x->bd)
                 : lbm::get_ops_f32_2d(x->M, x->energy, &x->of) && lbm::get_batch_ops_f32(x->M, x->energy, &x->bf);
@@ -526,11 +542,19 @@ int lbm_create_batch(lbm_ctx** out, int n_cases, const lbm_config* cfgs) {
   // case table and the work lists of node tiles
   if (e == cudaSuccess)
     e = x->precision == LBM_FP64 ? upload_cases(x, x->case_pd, x->case_itd) : upload_cases(x, x->case_pf, x->case_itf);
-  const int tl[3] = {64, 128, 256};
-  for (int t = 0; t < 3 && e == cudaSuccess; ++t) {
+  for (int t = 0; t < 6 && e == cudaSuccess; ++t) {
+    int tx = 0, ty = 0;
+    if (x->precision == LBM_FP64) x->bd.tile(2 * t, &tx, &ty);
+    else x->bf.tile(2 * t, &tx, &ty);
     std::vector<int2> tiles;
-    for (int c = 0; c < n_cases; ++c)
-      for (int n0 = 0; n0 < x->case_N[c]; n0 += tl[t]) tiles.push_back(make_int2(c, n0));
+    for (int c = 0; c < n_cases; ++c) {
+      if (ty == 0) {
+        for (int n0 = 0; n0 < x->case_N[c]; n0 += tx) tiles.push_back(make_int2(c, n0));
+      } else {
+        const int k = ((x->case_nx[c] + tx - 1) / tx) * ((x->case_ny[c] + ty - 1) / ty);
+        for (int q = 0; q < k; ++q) tiles.push_back(make_int2(c, q));
+      }
+    }
     x->ntiles[t] = (int)tiles.size();
     e = cudaMalloc(&x->tiles_dev[t], tiles.size() * sizeof(int2));
     if (e == cudaSuccess) e = cudaMemcpy(x->tiles_dev[t], tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice);
@@ -621,7 +645,7 @@ constexpr int kGraphSteps = 50;    // even: a replay returns to the same ping-po
 
 template <class R>
 static lbm::BatchArgs<R> batch_args(lbm_ctx* x, int cur) {
-  const int t = (x->variant % 6) / 2;
+  const int t = x->variant / 2;
   return lbm::BatchArgs<R>{(const lbm::CaseDev<R>*)x->cases_dev, x->tiles_dev[t], x->ntiles[t],
                            (const R*)x->pops[cur], (R*)x->pops[1 - cur], (const R*)x->phi, (const R*)x->Tfix,
                            (R*)x->mac, x->status};
@@ -629,7 +653,7 @@ static lbm::BatchArgs<R> batch_args(lbm_ctx* x, int cur) {
 
 template <class R>
 static int batch_grid(lbm_ctx* x, const lbm::BatchOps<R>& ops) {
-  const int nt = x->ntiles[(x->variant % 6) / 2];
+  const int nt = x->ntiles[x->variant / 2];
   if (x->variant % 2) return nt;
   const int g = x->sm_count * ops.occupancy(x->variant);
   return g < nt ? g : nt;
@@ -639,7 +663,7 @@ template <class R>
 static void batch_launch(lbm_ctx* x, const lbm::BatchOps<R>& ops, int cur, cudaStream_t s) {
   const lbm::BatchArgs<R> a = batch_args<R>(x, cur);
   const int grid = batch_grid(x, ops);
-  ops.pass(a, x->variant, grid, 0, s);
+  if (lbm::batch_two_pass(x->variant)) ops.pass(a, x->variant, grid, 0, s);
   ops.pass(a, x->variant, grid, 1, s);
 }
 
@@ -689,7 +713,7 @@ static int batch_steps(lbm_ctx* x, const lbm::BatchOps<R>& ops, int n) {
   for (; n > 0; --n) {
     const lbm::BatchArgs<R> a = batch_args<R>(x, x->cur);
     const int grid = batch_grid(x, ops);
-    timed(x, 0, [&] { ops.pass(a, x->variant, grid, 0, x->stream); });
+    if (lbm::batch_two_pass(x->variant)) timed(x, 0, [&] { ops.pass(a, x->variant, grid, 0, x->stream); });
     timed(x, 1, [&] { ops.pass(a, x->variant, grid, 1, x->stream); });
     x->cur = 1 - x->cur;
   }
@@ -1254,7 +1278,7 @@ void lbm_destroy(lbm_ctx* x) {
     if (b) cudaFree(b);
   drop_graphs(x);
   if (x->cases_dev) cudaFree(x->cases_dev);
-  for (int t = 0; t < 3; ++t)
+  for (int t = 0; t < 6; ++t)
     if (x->tiles_dev[t]) cudaFree(x->tiles_dev[t]);
   if (x->cap_stream) cudaStreamDestroy(x->cap_stream);
   for (cudaEvent_t ev : x->ev) cudaEventDestroy(ev);

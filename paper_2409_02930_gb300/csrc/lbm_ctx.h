@@ -68,8 +68,8 @@ struct lbm_ctx {
   std::vector<lbm::InletTables<double>> case_itd;
   std::vector<lbm::InletTables<float>> case_itf;
   void* cases_dev;                   // CaseDev<R>[n_cases]
-  int2* tiles_dev[3];                // work lists for tile lengths 64, 128, 256
-  int ntiles[3];
+  int2* tiles_dev[6];                // work lists of the variants' tile shapes (variant / 2)
+  int ntiles[6];
   lbm::BatchOps<double> bd;
   lbm::BatchOps<float> bf;
   int sm_count;

@@ -11,14 +11,9 @@
 // re-reads hit L2) and written once.
 #pragma once
 
-#include "lbm_twopass.cuh"
+#include "lbm_tile2d.cuh"
 
 namespace lbm {
-
-LBM_HD int modp(int v, int n) {
-  int r = v % n;
-  return r < 0 ? r + n : r;
-}
 
 template <int D, int M, bool EN>
 struct FusedLayout {

@@ -25,7 +25,9 @@ int configure(Kern kern, size_t smem, bool& done) {
 
 template <class R, int D, int M, bool EN>
 struct Launch {
-  static int grid(int N) { return (N + 255) / 256; }
+  // small lattices take small blocks, so that they spread over the SMs
+  static int block(int N) { return N < 152 * 512 ? 64 : 256; }
+  static int grid(int N) { return (N + block(N) - 1) / block(N); }
   // 3-D: the step split by lattice, NB = 32 nodes and one warp per lattice in a block
   static constexpr int NB = 32, L = M + 1 + (EN ? 1 : 0);
   template <bool AUX>
@@ -51,11 +53,11 @@ struct Launch {
   static constexpr int kMinB = sizeof(R) == 4 ? 2 : 1;
   static void macro(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
     if constexpr (D == 3) macro3<false>(p, it, a, nullptr, s);
-    else k_macro<R, D, M, EN><<<grid(p.N), 256, 0, s>>>(p, it, a);
+    else k_macro<R, D, M, EN><<<grid(p.N), block(p.N), 0, s>>>(p, it, a);
   }
   static void collide(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
     if constexpr (D == 3) collide3<false, kMinB>(p, it, a, nullptr, s);
-    else k_collide<R, D, M, EN><<<grid(p.N), 256, 0, s>>>(p, it, a);
+    else k_collide<R, D, M, EN><<<grid(p.N), block(p.N), 0, s>>>(p, it, a);
   }
   // fused step, shared-memory halo ring, tile TX x TY marching SEG planes
   template <int TX, int TY, int SEG>
@@ -68,6 +70,14 @@ struct Launch {
     dim3 g((p.nx + TX - 1) / TX, D == 3 ? (p.ny + TY - 1) / TY : (p.ny + SEG - 1) / SEG,
            D == 3 ? (p.nz + SEG - 1) / SEG : 1);
     kern<<<g, TX * TY, smem, s>>>(p, it, a);
+    return 0;
+  }
+  // tiles with the populations in registers
+  template <int TX, int TY, int MINB>
+  static int tile2d(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
+    if ((p.ny + TY - 1) / TY > 65535) return -1;
+    if constexpr (D == 2)
+      k_tile2d<R, M, EN, TX, TY, MINB><<<dim3((p.nx + TX - 1) / TX, (p.ny + TY - 1) / TY), TX * TY, 0, s>>>(p, it, a);
     return 0;
   }
   // pipelined 2-D step (cp.async staging), TX columns marching SEG rows
@@ -146,6 +156,9 @@ struct Launch {
         case 7: return staged<128>(p, it, a, s);
         case 8: return march2d_tma<32, 8, 1, 1>(p, it, a, s);
         case 9: return march2d_tma<64, 8, 1, 1>(p, it, a, s);
+        case 10: return tile2d<8, 4, 1>(p, it, a, s);
+        case 11: return tile2d<16, 8, sizeof(R) == 4 ? 3 : 1>(p, it, a, s);
+        case 12: return tile2d<32, 4, sizeof(R) == 4 ? 3 : 1>(p, it, a, s);
         default: return -1;
       }
     } else {
@@ -161,14 +174,14 @@ struct Launch {
       }
     }
   }
-  static constexpr int n_variants = (D == 2) ? 10 : 6;
+  static constexpr int n_variants = (D == 2) ? 13 : 6;
   static void init(const Params<R>& p, const double* X, const double* T, const double* P, const double* U,
                    double cvel, double RU, R* dst, const R* phi, cudaStream_t s) {
-    k_init<R, D, M, EN><<<grid(p.N), 256, 0, s>>>(p, X, T, P, U, cvel, RU, dst, phi);
+    k_init<R, D, M, EN><<<grid(p.N), block(p.N), 0, s>>>(p, X, T, P, U, cvel, RU, dst, phi);
   }
   static void moments(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, int which, double cvel,
                       double* out, cudaStream_t s) {
-    k_moments<R, D, M, EN><<<grid(p.N), 256, 0, s>>>(p, it, a, which, cvel, out);
+    k_moments<R, D, M, EN><<<grid(p.N), block(p.N), 0, s>>>(p, it, a, which, cvel, out);
   }
   static constexpr bool has_react = (D == 3 && M == 6 && EN);
   static void react_macro(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, const ReactArgs& ra,

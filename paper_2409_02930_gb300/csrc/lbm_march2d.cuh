@@ -16,7 +16,7 @@
 // missing populations are reservoir equilibria computed on the fly).
 #pragma once
 
-#include "lbm_twopass.cuh"
+#include "lbm_tile2d.cuh"
 #include "lbm_tma.cuh"
 
 namespace lbm {

@@ -85,9 +85,9 @@ void to_precision(const lbm::Params<double>& d, lbm::Params<R>& r, const lbm::In
 
 template <class R, int M, bool EN>
 void launch(const lbm::Params<R>& p, const lbm::InletTables<R>& it, const lbm::StepArgs<R>& a, cudaStream_t s) {
-  const int grid = (p.N + 255) / 256;
-  lbm::k_macro<R, 2, M, EN><<<grid, 256, 0, s>>>(p, it, a);
-  lbm::k_collide<R, 2, M, EN><<<grid, 256, 0, s>>>(p, it, a);
+  const int block = p.N < 152 * 512 ? 64 : 256, grid = (p.N + block - 1) / block;
+  lbm::k_macro<R, 2, M, EN><<<grid, block, 0, s>>>(p, it, a);
+  lbm::k_collide<R, 2, M, EN><<<grid, block, 0, s>>>(p, it, a);
 }
 
 template <class R>
