@@ -223,6 +223,11 @@ __global__ void __launch_bounds__(128) k_adj_macro(Params<B> p, AdjArgs<B> a) {
     state_reverse<B, M, EN>(p, s, mo.sg, S_, sa_, sf_, jf_, sg_);
     a.phibar[n] += (double)phi_;
   }
+  // every load before the first store: the two arrays may alias for the
+  // compiler, and load-store pairs in turn cost a round trip each
+  B v[L * 9];
+#pragma unroll
+  for (int e = 0; e < L * 9; ++e) v[e] = a.Pbar[(size_t)(unsigned)e * N + n];
   Unroll<0, 9>::run([&](auto ic) {
     constexpr int i = decltype(ic)::value;
     constexpr int cx = c_of<2>(i, 0), cy = c_of<2>(i, 1);
@@ -236,13 +241,12 @@ __global__ void __launch_bounds__(128) k_adj_macro(Params<B> p, AdjArgs<B> a) {
     if (cy < 0) jc -= jf_[1];
 #pragma unroll
     for (int l = 0; l < L; ++l) {
-      B* q = a.Pbar + (size_t)(unsigned)(l * 9 + i) * N + n;
-      const B v = *q + (l < M ? sa_[l < M ? l : 0] : (l == M ? sf_ + jc : sg_));
+      const B t = v[l * 9 + i] + (l < M ? sa_[l < M ? l : 0] : (l == M ? sf_ + jc : sg_));
       if (h == SRC_GHOST) {
-        *q = v;
+        a.Pbar[(size_t)(unsigned)(l * 9 + i) * N + n] = t;
         a.lam0[(size_t)(unsigned)(l * 9 + 8 - i) * N + n] = B(0);    // leaves through the face
       } else {
-        a.lam0[(size_t)((unsigned)(l * 9) + isrc) * N + src] = v;
+        a.lam0[(size_t)((unsigned)(l * 9) + isrc) * N + src] = t;
       }
     }
   });
@@ -268,10 +272,12 @@ __global__ void __launch_bounds__(32) k_adj_ghost(Params<B> p, InletTables<B> it
     const int nb = (side == 0 ? 0 : p.nx - 1) + p.nx * y, xa = side == 0 ? 1 : p.nx - 2, na = xa + p.nx * y;
     Site<B, 2> sa;
     sa.init(p, xa, y, 0);
-    B s0 = B(0), j[2] = {B(0), B(0)};
+    B s0 = B(0), j[2] = {B(0), B(0)}, lam[9];
     Unroll<0, 9>::run([&](auto ic) {
       constexpr int i = decltype(ic)::value;
-      const B f = a.f[(size_t)(M * 9 + i) * N + sa.source(c_of<2>(i, 0), c_of<2>(i, 1), 0)];
+      const size_t at = (size_t)(M * 9 + i) * N + sa.source(c_of<2>(i, 0), c_of<2>(i, 1), 0);
+      const B f = a.f[at];
+      lam[i] = a.lam0[at];
       s0 += f;
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
@@ -308,7 +314,7 @@ __global__ void __launch_bounds__(32) k_adj_ghost(Params<B> p, InletTables<B> it
     Unroll<0, 9>::run([&](auto ic) {
       constexpr int i = decltype(ic)::value;
       constexpr int cx = c_of<2>(i, 0), cy = c_of<2>(i, 1);
-      a.lam0[(size_t)(M * 9 + i) * N + sa.source(cx, cy, 0)] += s_ + r * (B(cx) * acc[0] + B(cy) * acc[1]);
+      a.lam0[(size_t)(M * 9 + i) * N + sa.source(cx, cy, 0)] = lam[i] + (s_ + r * (B(cx) * acc[0] + B(cy) * acc[1]));
     });
     a.phibar[na] += (double)((acc[0] * gh.u[0].v + acc[1] * gh.u[1].v) / pa);
     a.phibar[nb] += (double)acc[2];
