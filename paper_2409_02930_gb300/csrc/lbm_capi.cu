@@ -228,16 +228,13 @@ static int setup_surface(lbm_ctx* x, const lbm_config* c) {
     int nr = 0;
     for (int a = 0; a < c->M + c->S; ++a) {
       const double v = a < c->M ? c->nu_gas[k * c->M + a] : c->nu_surf[k * c->S + (a - c->M)];
-      if (a < c->M) h.nu_g[k][a] = v;
-      else h.nu_s[k][a - c->M] = v;
-      h.nu_all[k][a] = v;
       if (v != 0) {
         if (h.npart[k] >= 8) return fail(nullptr, LBM_ERR_ARG, "at most 8 species take part in one surface step");
         h.pidx[k][h.npart[k]] = a;
         h.pnu[k][h.npart[k]] = v;
+        h.pnuf[k][h.npart[k]] = (float)v;
         h.npart[k]++;
         h.sr_k[a][h.nsr[a]] = k;
-        h.sr_nuf[a][h.nsr[a]] = (float)v;
         h.sr_nud[a][h.nsr[a]] = v;
         h.nsr[a]++;
       }

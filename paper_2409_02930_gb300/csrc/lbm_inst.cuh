@@ -189,7 +189,13 @@ struct Launch {
     if constexpr (has_react) {
       R* aux = a.mac + (size_t)(2 * D + M) * p.N;
       macro3<true>(p, it, a, aux, s);
-      k_source<R, M><<<(p.N + 127) / 128, 128, 0, s>>>(p.N, aux, a.phi, a.status, ra);
+      if (p.N <= source_warp_nodes) {
+        k_source_warp<R, M><<<p.N, 32, 0, s>>>(p.N, aux, a.phi, a.status, ra);
+      } else if (p.N <= source_wide_nodes) {
+        k_source<R, M, 1><<<(p.N + 127) / 128, 128, 0, s>>>(p.N, aux, a.phi, a.status, ra);
+      } else {
+        k_source<R, M, sizeof(R) == 4 ? 10 : 8><<<(p.N + 127) / 128, 128, 0, s>>>(p.N, aux, a.phi, a.status, ra);
+      }
     }
   }
   static void react_collide(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, const ReactArgs& ra,

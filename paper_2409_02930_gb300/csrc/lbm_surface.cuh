@@ -27,15 +27,12 @@ constexpr double R_UNIV_DEV = 8.314462618;    // J/(mol K)
 // mol/m^2); reactant lists hold the integer mass-action orders.
 struct MechDev {
   int M, S, R;
-  double nu_g[RMAX][MMAX];
-  double nu_s[RMAX][SMAX];
-  double nu_all[RMAX][MMAX + SMAX];
   int npart[RMAX];                   // species taking part in each step (nonzero stoichiometry)
   int pidx[RMAX][8];
   double pnu[RMAX][8];
+  float pnuf[RMAX][8];
   int nsr[MMAX + SMAX];               // steps in which each species takes part
   int sr_k[MMAX + SMAX][RMAX];
-  float sr_nuf[MMAX + SMAX][RMAX];
   double sr_nud[MMAX + SMAX][RMAX];
   int nre[RMAX];                     // reactants of each step
   int ridx[RMAX][4];
@@ -58,10 +55,10 @@ struct MechDev {
 
 constexpr double FARADAY_DEV = 96485.33212;   // C/mol
 
-// stoichiometric coefficient of species i in its q-th step, in the Jacobian's precision
-template <class RK> __device__ __forceinline__ RK sr_nu(const MechDev& mc, int i, int q);
-template <> __device__ __forceinline__ float sr_nu<float>(const MechDev& mc, int i, int q) { return mc.sr_nuf[i][q]; }
-template <> __device__ __forceinline__ double sr_nu<double>(const MechDev& mc, int i, int q) { return mc.sr_nud[i][q]; }
+// stoichiometric coefficient of the q-th species of step k, in the Jacobian's precision
+template <class RK> __device__ __forceinline__ RK pnu_of(const MechDev& mc, int k, int q);
+template <> __device__ __forceinline__ float pnu_of<float>(const MechDev& mc, int k, int q) { return mc.pnuf[k][q]; }
+template <> __device__ __forceinline__ double pnu_of<double>(const MechDev& mc, int k, int q) { return mc.pnu[k][q]; }
 
 __device__ __forceinline__ double ipow(double x, int n) {
   double r = 1.0;
@@ -81,126 +78,190 @@ __device__ __forceinline__ double ipow(double x, int n) {
 // contraction of the steps slows down or a step is shortened, when they are
 // rebuilt at the current iterate.  The FP64 residual fixes the root, so every variant
 // converges to the same FP64 solution.
+//
+// What bounds it: the FP64 pipe and the latency of the per-thread work arrays
+// in local memory.  FP64 divisions are kept out of the loops (one 1/(R_U T)
+// per node; the rates' derivatives are products without the factor they are
+// taken by, so no rate is divided by a concentration), the concentrations
+// follow the extents by increments, and the tests that only steer the
+// iteration compare high words as integers.  The factorisation is unrolled
+// over the pivots with the pivot row in registers and the triangular solves
+// over both indices with the right-hand side in registers, so each multiply-
+// add touches local memory once (twice while factorising) instead of twice
+// (three times).
 template <int M, class RK>
 __device__ void surface_source_dev(const MechDev& mc, double T, const double* rho_a, double phi, const double* Xs0,
                                    double* rhodot, double* Xs1, double& dU, double& current, double dphi,
                                    int* status) {
   const int S = mc.S, Rn = mc.R, NS = M + mc.S;
-  double c0[MMAX + SMAX], kr[RMAX], xi[RMAX];
+  constexpr int NSX = MMAX + SMAX;
+  double c0[NSX], d[NSX], kr[RMAX], xi[RMAX];
+  const double inv_RT = 1.0 / (R_UNIV_DEV * T);
   for (int a = 0; a < M; ++a) c0[a] = rho_a[a] / mc.m[a];
   for (int s = 0; s < S; ++s) c0[M + s] = mc.gamma * Xs0[s];
+  for (int i = 0; i < NS; ++i) d[i] = 0.0;
   for (int k = 0; k < Rn; ++k) {
-    kr[k] = mc.A[k] * exp(-mc.Ea[k] / (R_UNIV_DEV * T));
+    double v = mc.A[k] * exp(-mc.Ea[k] * inv_RT);
     // TPB step: rate per unit TPB length, extent counted per unit surface
-    if (mc.edge[k])
-      kr[k] *= (mc.l_tpb / mc.a_s) * exp(mc.beta_ct * mc.nel[k] * FARADAY_DEV * dphi / (R_UNIV_DEV * T));
+    if (mc.edge[k]) v *= (mc.l_tpb / mc.a_s) * exp(mc.beta_ct * mc.nel[k] * FARADAY_DEV * dphi * inv_RT);
+    kr[k] = v;
     xi[k] = 0.0;
   }
   const double scale = mc.a_s / phi;     // gas concentration change per extent
+  const RK rscale = RK(scale);
   // J = I - U V with U = dt dr/dc (R x NS, the reactants of each step) and
   // V = diag(scale) nu^T (NS x R); by the Woodbury identity
   // J^-1 b = b + U K^-1 V b with K = I - V U (NS x NS), whose LU factors and U
   // are kept while the iteration reuses them.
-  constexpr int NSX = MMAX + SMAX;
   RK LU[NSX][NSX];
   RK uk[RMAX][4];
-  int swp[NSX];
+  int perm[NSX];
   bool refresh = true, converged = false;
   double prev = 0.0;
   for (int it = 0; it < 40; ++it) {
-    double c[MMAX + SMAX], r[RMAX];
-    // c = c0 + (scaled) nu^T xi, over the few species of each step
-    double d[MMAX + SMAX];
-    for (int i = 0; i < NS; ++i) d[i] = 0.0;
-    for (int k = 0; k < Rn; ++k)
-      for (int j = 0; j < mc.npart[k]; ++j) d[mc.pidx[k][j]] += mc.pnu[k][j] * xi[k];
-    for (int i = 0; i < NS; ++i) c[i] = c0[i] + (i < M ? scale : 1.0) * d[i];
-    for (int k = 0; k < Rn; ++k) {
-      double v = kr[k];
-      for (int j = 0; j < mc.nre[k]; ++j) v *= ipow(fmax(c[mc.ridx[k][j]], 0.0), mc.rord[k][j]);
-      r[k] = v;
+    double c[NSX], pos[NSX];
+    RK b[RMAX], w[NSX];
+    for (int i = 0; i < NS; ++i) {
+      c[i] = c0[i] + (i < M ? scale : 1.0) * d[i];
+      pos[i] = fmax(c[i], 0.0);
+      w[i] = RK(0);
     }
-    if (refresh) {
-      // U entries dt r_k ord / c_j of the reactants j of each step, and K = I - V U
+    if (refresh)
       for (int i = 0; i < NS; ++i)
         for (int j = 0; j < NS; ++j) LU[i][j] = (i == j) ? RK(1) : RK(0);
-      for (int k = 0; k < Rn; ++k)
-        for (int j = 0; j < mc.nre[k]; ++j) {
+    for (int k = 0; k < Rn; ++k) {
+      // rate r = k prod c^o; where the Jacobian is rebuilt also its derivatives
+      // u_j = dt k o_j c_j^(o_j - 1) prod of the others (zero where c_j <= 0)
+      const int nre = mc.nre[k];
+      double f[4], g[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        f[j] = g[j] = 1.0;
+        if (j < nre) {
+          const double v = pos[mc.ridx[k][j]];
+          const int o = mc.rord[k][j];
+          if (o > 1) g[j] = ipow(v, o - 1);
+          f[j] = o > 1 ? g[j] * v : v;
+        }
+      }
+      double r = kr[k] * f[0];
+      if (nre > 1) r *= f[1];
+      if (nre > 2) r *= f[2] * f[3];
+      const RK bk = RK(-(xi[k] - mc.dt * r));
+      b[k] = bk;
+      for (int q = 0; q < mc.npart[k]; ++q) {
+        const int i = mc.pidx[k][q];
+        w[i] += (i < M ? rscale : RK(1)) * pnu_of<RK>(mc, k, q) * bk;
+      }
+      if (refresh) {
+        const double dk = mc.dt * kr[k];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (j >= nre) continue;
           const int jj = mc.ridx[k][j];
-          const RK u = c[jj] > 0.0 ? RK(mc.dt * r[k] * mc.rord[k][j] / c[jj]) : RK(0);
-          uk[k][j] = u;
+          double u = dk * g[j];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (e != j && e < nre) u *= f[e];
+          const RK ur = c[jj] > 0.0 ? RK(u * mc.rord[k][j]) : RK(0);
+          uk[k][j] = ur;
           for (int q = 0; q < mc.npart[k]; ++q) {
             const int i = mc.pidx[k][q];
-            LU[i][jj] -= RK((i < M ? scale : 1.0) * mc.pnu[k][q]) * u;
+            LU[i][jj] -= (i < M ? rscale : RK(1)) * pnu_of<RK>(mc, k, q) * ur;
           }
         }
-      // LU factors of K with partial pivoting (row swaps recorded in swp)
-      for (int cc = 0; cc < NS; ++cc) {
+      }
+    }
+    if (refresh) {
+      // LU factors of K with partial pivoting (row order recorded in perm)
+      for (int i = 0; i < NS; ++i) perm[i] = i;
+#pragma unroll
+      for (int cc = 0; cc < NSX; ++cc) {
+        if (cc >= NS) break;
         int pv = cc;
-        for (int k = cc + 1; k < NS; ++k)
-          if (fabs(LU[k][cc]) > fabs(LU[pv][cc])) pv = k;
-        swp[cc] = pv;
-        if (pv != cc)
-          for (int l = 0; l < NS; ++l) {
-            RK t = LU[cc][l];
-            LU[cc][l] = LU[pv][l];
-            LU[pv][l] = t;
+        RK best = fabs(LU[cc][cc]);
+        for (int k = cc + 1; k < NS; ++k) {
+          const RK v = fabs(LU[k][cc]);
+          if (v > best) {
+            best = v;
+            pv = k;
           }
-        const RK inv = RK(1) / LU[cc][cc];
+        }
+        RK prow[NSX];
+        const int pp = perm[pv];
+        perm[pv] = perm[cc];
+        perm[cc] = pp;
+#pragma unroll
+        for (int l = 0; l < NSX; ++l) {
+          if (l >= NS) break;
+          const RK t = LU[cc][l];
+          prow[l] = LU[pv][l];
+          if (pv != cc) {
+            LU[pv][l] = t;
+            LU[cc][l] = prow[l];
+          }
+        }
+        const RK inv = RK(1) / prow[cc];
         for (int k = cc + 1; k < NS; ++k) {
           const RK f = LU[k][cc] * inv;
           LU[k][cc] = f;
-          for (int l = cc + 1; l < NS; ++l) LU[k][l] -= f * LU[cc][l];
+#pragma unroll
+          for (int l = cc + 1; l < NSX; ++l) {
+            if (l >= NS) break;
+            LU[k][l] -= f * prow[l];
+          }
         }
+        LU[cc][cc] = inv;                              // the solves multiply by the pivot's reciprocal
       }
       refresh = false;
     }
     // solve J dxi = -F:  w = V b, K z = w, dxi = b + U z
-    RK b[RMAX], w[NSX];
-    for (int k = 0; k < Rn; ++k) b[k] = RK(-(xi[k] - mc.dt * r[k]));
-    for (int i = 0; i < NS; ++i) w[i] = RK(0);
-    for (int k = 0; k < Rn; ++k)
-      for (int q = 0; q < mc.npart[k]; ++q) {
-        const int i = mc.pidx[k][q];
-        w[i] += RK((i < M ? scale : 1.0) * mc.pnu[k][q]) * b[k];
+    {
+      RK y[NSX];
+#pragma unroll
+      for (int k = 0; k < NSX; ++k) {
+        if (k >= NS) break;
+        y[k] = w[perm[k]];
+#pragma unroll
+        for (int l = 0; l < k; ++l) y[k] -= LU[k][l] * y[l];
       }
-    for (int cc = 0; cc < NS; ++cc)
-      if (swp[cc] != cc) {
-        RK t = w[cc];
-        w[cc] = w[swp[cc]];
-        w[swp[cc]] = t;
+#pragma unroll
+      for (int k = NSX - 1; k >= 0; --k) {
+        if (k >= NS) continue;
+#pragma unroll
+        for (int l = k + 1; l < NSX; ++l) {
+          if (l >= NS) break;
+          y[k] -= LU[k][l] * y[l];
+        }
+        y[k] *= LU[k][k];
+        w[k] = y[k];
       }
-    for (int k = 1; k < NS; ++k)
-      for (int l = 0; l < k; ++l) w[k] -= LU[k][l] * w[l];
-    for (int k = NS - 1; k >= 0; --k) {
-      RK s2 = w[k];
-      for (int l = k + 1; l < NS; ++l) s2 -= LU[k][l] * w[l];
-      w[k] = s2 / LU[k][k];
     }
-    double dxi[RMAX];
+    double dd[NSX], dxi[RMAX];
+    for (int i = 0; i < NS; ++i) dd[i] = 0.0;
     for (int k = 0; k < Rn; ++k) {
       RK x = b[k];
       for (int j = 0; j < mc.nre[k]; ++j) x += uk[k][j] * w[mc.ridx[k][j]];
       dxi[k] = (double)x;
+      for (int j = 0; j < mc.npart[k]; ++j) dd[mc.pidx[k][j]] += mc.pnu[k][j] * dxi[k];
     }
     // steps that would take a non-negative concentration below zero are shortened
     double alpha = 1.0;
-    {
-      double dd[MMAX + SMAX];
-      for (int i = 0; i < NS; ++i) dd[i] = 0.0;
-      for (int k = 0; k < Rn; ++k)
-        for (int j = 0; j < mc.npart[k]; ++j) dd[mc.pidx[k][j]] += mc.pnu[k][j] * dxi[k];
-      for (int i = 0; i < NS; ++i) {
-        const double di = dd[i] * (i < M ? scale : 1.0);
-        if (c[i] >= 0.0 && c[i] + di < 0.0) alpha = fmin(alpha, 0.9 * c[i] / (-di));
-      }
+    for (int i = 0; i < NS; ++i) {
+      const double di = dd[i] * (i < M ? scale : 1.0);
+      if (c[i] >= 0.0 && c[i] + di < 0.0) alpha = fmin(alpha, 0.9 * c[i] / (-di));
     }
-    double dmax = 0.0, xmax = 0.0;
+    // largest step and extent, by the high words (20 mantissa bits: they only
+    // decide when to stop and when to rebuild)
+    int dtop = 0, xtop = 0;
     for (int k = 0; k < Rn; ++k) {
-      xi[k] += alpha * dxi[k];
-      dmax = fmax(dmax, fabs(alpha * dxi[k]));
-      xmax = fmax(xmax, fabs(xi[k]));
+      const double st = alpha * dxi[k];
+      xi[k] += st;
+      dtop = max(dtop, __double2hiint(st) & 0x7fffffff);
+      xtop = max(xtop, __double2hiint(xi[k]) & 0x7fffffff);
     }
+    for (int i = 0; i < NS; ++i) d[i] += alpha * dd[i];
+    const double dmax = __hiloint2double(dtop, 0), xmax = __hiloint2double(xtop, 0);
     if (alpha == 1.0 && dmax <= 1e-14 * (xmax + 1e-300)) {
       converged = true;
       break;
@@ -246,8 +307,8 @@ struct ReactArgs {
 
 // Surface source of every node, from the species sums and temperatures that
 // the macro-field pass left in aux ([M + 1][N]).
-template <class R, int M>
-__global__ void __launch_bounds__(128) k_source(int N, const R* __restrict__ aux, const R* __restrict__ phi,
+template <class R, int M, int MINB>
+__global__ void __launch_bounds__(128, MINB) k_source(int N, const R* __restrict__ aux, const R* __restrict__ phi,
                                                 int* status, ReactArgs ra) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
@@ -262,6 +323,221 @@ __global__ void __launch_bounds__(128) k_source(int N, const R* __restrict__ aux
   ra.src[(size_t)M * N + n] = dU;
   ra.src[(size_t)(M + 1) * N + n] = cur;
   for (int k = 0; k < mc.S; ++k) ra.Xs_out[(size_t)k * N + n] = Xs1[k];
+}
+
+// Which form a lattice of N nodes takes.  A warp per node up to 2048 nodes
+// (FP64 12 x 2 x 2: 157 us per reactive step against 380 us with a thread per
+// node; 8192 nodes FP32 376 against 303, so the line lies below 152 SMs x a few
+// warps).  Above it a thread per node: without a register limit while the
+// threads do not fill the GPU (8192 nodes FP32 303 us per step at 222
+// registers, 332 at 48), then limited to 48 (FP32) or 64 (FP64) registers, so
+// that more threads hide the latency of the work arrays (524,288 nodes FP32
+// 5.58 -> 4.45 ms per step).
+constexpr int source_warp_nodes = 2048;
+constexpr int source_wide_nodes = 152 * 128 * 2;
+
+// The same source with one warp per node, for lattices too small to fill the
+// GPU with a thread per node: there the time is the latency of one node's
+// Newton iteration, whose loops a warp runs side by side.  Lane k holds
+// reaction k (rate, extent, Jacobian entries), lane i species i
+// (concentration, row i of K in registers); rows are eliminated in pivot
+// order without being moved (the pivot lane's row is broadcast by shuffles),
+// so no work array is indexed dynamically.  The iteration, its thresholds and
+// the precision of every quantity are those of surface_source_dev; sums run
+// over a species' steps in the same order, and the concentrations follow the
+// extents by increments.  12 x 2 x 2 anode in FP64: see the figures above.
+template <class RK, int M>
+__global__ void __launch_bounds__(32) k_source_warp(int N, const RK* __restrict__ aux, const RK* __restrict__ phi,
+                                                    int* status, ReactArgs ra) {
+  constexpr int NSX = MMAX + SMAX;
+  constexpr unsigned FULL = 0xffffffffu;
+  __shared__ double s_nu[RMAX][NSX], s_c[32], s_x[32];
+  __shared__ unsigned char s_k[RMAX][NSX];
+  __shared__ RK s_b[32], s_u[RMAX][4], s_K[NSX][NSX + 1];
+  const int lane = threadIdx.x;
+  const MechDev& mc = *ra.mech;
+  const int S = mc.S, Rn = mc.R, NS = M + S;
+  const bool sp = lane < NS, re = lane < Rn;
+  const int nq = sp ? mc.nsr[lane] : 0;
+  for (int q = 0; q < nq; ++q) {
+    s_k[q][lane] = (unsigned char)mc.sr_k[lane][q];
+    s_nu[q][lane] = mc.sr_nud[lane][q];
+  }
+  int nre = 0, ri[4], ro[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) ri[j] = ro[j] = 0;
+  if (re) {
+    nre = mc.nre[lane];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (j < nre) {
+        ri[j] = mc.ridx[lane][j];
+        ro[j] = mc.rord[lane][j];
+      }
+  }
+  const int n = blockIdx.x;
+  const double ph = (double)phi[n], T = (double)aux[(size_t)M * N + n];
+  const double dphi = mc.dphi_field ? mc.dphi_field[n] : mc.dphi;
+  const double scale = lane < M ? mc.a_s / ph : 1.0;       // concentration change per extent of species `lane`
+  double c0 = 0.0, Xs0 = 0.0;
+  if (lane < M) c0 = (double)(aux[(size_t)lane * N + n] / phi[n]) / mc.m[lane];
+  else if (sp) {
+    Xs0 = ra.Xs_in[(size_t)(lane - M) * N + n];
+    c0 = mc.gamma * Xs0;
+  }
+  double kr = 0.0;
+  const bool edge = re && mc.edge[lane];
+  if (re) {
+    kr = mc.A[lane] * exp(-mc.Ea[lane] / (R_UNIV_DEV * T));
+    if (edge) kr *= (mc.l_tpb / mc.a_s) * exp(mc.beta_ct * mc.nel[lane] * FARADAY_DEV * dphi / (R_UNIV_DEV * T));
+  }
+  double xi = 0.0, d = 0.0;
+  RK row[NSX], inv[NSX], uk[4];
+  int pl[NSX], mine = 0;                                    // pivot lanes, and the step in which this row pivots
+#pragma unroll
+  for (int j = 0; j < 4; ++j) uk[j] = RK(0);
+  bool refresh = true, converged = false;
+  double prev = 0.0;
+  for (int it = 0; it < 40; ++it) {
+    const double c = c0 + scale * d;
+    s_c[lane] = c;
+    __syncwarp();
+    double r = kr;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (j < nre) r *= ipow(fmax(s_c[ri[j]], 0.0), ro[j]);
+    const RK b = RK(-(xi - mc.dt * r));
+    s_b[lane] = b;
+    if (refresh) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (j < nre) {
+          const double cj = s_c[ri[j]];
+          uk[j] = cj > 0.0 ? RK(mc.dt * r * ro[j] / cj) : RK(0);
+        }
+        s_u[lane][j] = uk[j];
+      }
+    }
+    __syncwarp();
+    if (refresh) {
+      // row `lane` of K = I - V U
+      if (sp) {
+        for (int j = 0; j < NS; ++j) s_K[lane][j] = (j == lane) ? RK(1) : RK(0);
+        for (int q = 0; q < nq; ++q) {
+          const int k = s_k[q][lane];
+          const RK v = RK(scale * s_nu[q][lane]);
+          const int m = mc.nre[k];
+          for (int j = 0; j < m; ++j) s_K[lane][mc.ridx[k][j]] -= v * s_u[k][j];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < NSX; ++j) row[j] = (sp && j < NS) ? s_K[lane][j] : RK(0);
+      // LU with partial pivoting: the largest entry of the column among the
+      // rows not yet taken (compared in single precision, lane in the low bits)
+      bool taken = !sp;
+      mine = NSX;
+#pragma unroll
+      for (int cc = 0; cc < NSX; ++cc) {
+        if (cc >= NS) break;
+        const unsigned bits = (__float_as_uint((float)fabs(row[cc])) & ~31u) | 32u;
+        const unsigned key = taken ? 0u : (bits | (unsigned)lane);
+        pl[cc] = (int)(__reduce_max_sync(FULL, key) & 31u);
+        if (lane == pl[cc]) {
+          taken = true;
+          mine = cc;
+        }
+        inv[cc] = RK(1) / __shfl_sync(FULL, row[cc], pl[cc]);
+        const RK f = row[cc] * inv[cc];
+#pragma unroll
+        for (int j = cc + 1; j < NSX; ++j) {
+          if (j >= NS) break;
+          const RK pj = __shfl_sync(FULL, row[j], pl[cc]);
+          if (!taken) row[j] -= f * pj;
+        }
+        if (!taken) row[cc] = f;
+      }
+      refresh = false;
+    }
+    // solve J dxi = -F:  w = V b, K z = w, dxi = b + U z
+    RK w = RK(0);
+    for (int q = 0; q < nq; ++q) w += RK(scale * s_nu[q][lane]) * s_b[s_k[q][lane]];
+#pragma unroll
+    for (int cc = 0; cc < NSX; ++cc) {
+      if (cc >= NS) break;
+      const RK wp = __shfl_sync(FULL, w, pl[cc]);
+      if (sp && mine > cc) w -= row[cc] * wp;
+    }
+    RK z = RK(0);
+#pragma unroll
+    for (int cc = NSX - 1; cc >= 0; --cc) {
+      if (cc >= NS) continue;
+      const RK xc = __shfl_sync(FULL, w, pl[cc]) * inv[cc];
+      if (sp && mine < cc) w -= row[cc] * xc;
+      if (lane == cc) z = xc;
+    }
+    double dxi = 0.0;
+    {
+      RK x = b;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const RK zj = __shfl_sync(FULL, z, ri[j]);
+        if (j < nre) x += uk[j] * zj;
+      }
+      if (re) dxi = (double)x;
+    }
+    s_x[lane] = dxi;
+    __syncwarp();
+    // steps that would take a non-negative concentration below zero are shortened
+    double dd = 0.0;
+    for (int q = 0; q < nq; ++q) dd += s_nu[q][lane] * s_x[s_k[q][lane]];
+    const double di = dd * scale;
+    double alpha = (sp && c >= 0.0 && c + di < 0.0) ? fmin(1.0, 0.9 * c / (-di)) : 1.0;
+    if (__any_sync(FULL, alpha < 1.0)) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) alpha = fmin(alpha, __shfl_xor_sync(FULL, alpha, o));
+    } else {
+      alpha = 1.0;
+    }
+    xi += alpha * dxi;
+    d += alpha * dd;
+    // largest step and extent, by the high words (20 mantissa bits: they only
+    // decide when to stop and when to rebuild)
+    auto top = [&](double v) {
+      return __hiloint2double((int)__reduce_max_sync(FULL, (unsigned)__double2hiint(v) & 0x7fffffffu), 0);
+    };
+    const double dmax = top(alpha * dxi), xmax = top(xi);
+    if (alpha == 1.0 && dmax <= 1e-14 * (xmax + 1e-300)) {
+      converged = true;
+      break;
+    }
+    refresh = (alpha < 1.0) || (it > 0 && dmax > 0.25 * prev);
+    prev = dmax;
+  }
+  if (!converged && lane == 0) flag(status, 4);
+  s_x[lane] = re ? xi : 0.0;
+  __syncwarp();
+  double dn = 0.0;                                          // moles produced per unit surface, nu^T xi
+  for (int q = 0; q < nq; ++q) dn += s_nu[q][lane] * s_x[s_k[q][lane]];
+  double dUs = 0.0, ne = edge ? mc.nel[lane] * xi : 0.0;
+  if (lane < M) {
+    ra.src[(size_t)lane * N + n] = mc.a_s * mc.m[lane] * dn;
+  } else if (sp) {
+    ra.Xs_out[(size_t)(lane - M) * N + n] = Xs0 + dn / mc.gamma;
+    dUs = mc.a_s * dn * (mc.Us0[lane - M] + mc.cvs[lane - M] * R_UNIV_DEV * (T - mc.T_thermo));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    dUs += __shfl_xor_sync(FULL, dUs, o);
+    ne += __shfl_xor_sync(FULL, ne, o);
+  }
+  if (lane == 0) {
+    const double current = FARADAY_DEV * mc.a_s * ne / mc.dt;
+    double Usrc = 0.0;
+    if (mc.l_tpb > 0.0)
+      Usrc = ((mc.a_s / mc.l_tpb) * current * current * mc.resist * mc.dx - fabs(dphi) * current) * mc.dt;
+    ra.src[(size_t)M * N + n] = (-dUs + Usrc) / mc.cvel2;
+    ra.src[(size_t)(M + 1) * N + n] = current;
+  }
 }
 
 }  // namespace lbm
