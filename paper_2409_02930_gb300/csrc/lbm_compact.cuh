@@ -313,12 +313,11 @@ LBM_HD R relax_dirs(Get&& get, int cz, R keep, const R (&m)[9], const R* ex, Put
   return acc;
 }
 
-template <class R, int D, bool EXTRA, class PullF>
-LBM_HD R relax_slice(const PullF& pf, int l, int cz, R keep, const R (&m)[9], const R* ex, R* __restrict__ dn,
-                     unsigned N) {
-  constexpr int Q = Lat<D>::Q;
-  return relax_dirs<R, D, EXTRA>([&](int i) { return pf.get(l, i); }, cz, keep, m, ex,
-                                 [&](int i, const R& v) { dn[(size_t)(unsigned)(l * Q + i) * N] = v; });
+// The same for lattice l of a D2Q9 node: put(l, i, value).
+template <class R, int D, bool EXTRA, class PullF, class Put>
+LBM_HD R relax_slice(const PullF& pf, int l, R keep, const R (&m)[9], const R* ex, Put&& put) {
+  return relax_dirs<R, D, EXTRA>([&](int i) { return pf.get(l, i); }, 0, keep, m, ex,
+                                 [&](int i, const R& v) { put(l, i, v); });
 }
 
 // Axis moments of one species: E (moving with w), S (moving with w + v) and
@@ -365,14 +364,15 @@ struct SpeciesAxes {
 };
 
 // Relaxation target of species a in scaled moments at z order k (Eq. 21, Eq. 25):
-//   T_a = cE E_a - gE (E_a - K_a) - gd d_a + qY sum_{b != a} invDmm_ab d_b
+//   T_a = cE E_a - gE (E_a - K_a) + sum_b X_ab d_b,  X_ab = qY invDmm_ab, X_aa = -gd
 // with d_b = sa_b (S_b - E_b), gd = (1 - beta_a)/tau^k_a, gE = gd sa_a,
 // qY = (1 - beta_a) Y_a C and cE = 2 beta_a sa_a (+ the source of Eq. 89).
 template <class R, int D>
 struct SpeciesTarget {
-  R cE, gE, gd, qY, th;
+  R cE, gE, th;
+  // the part without the coupling
   template <int k>
-  LBM_HD R entry(const SpeciesAxes<R, D>& ax, const R* w, int i, int j, R dl, R sum) const {
+  LBM_HD R entry(const SpeciesAxes<R, D>& ax, const R* w, int i, int j) const {
     constexpr bool Z = (D == 3) && k > 0;
     R Em = ax.E[0].m[i];
     if (j > 0) Em = (i > 0) ? Em * ax.E[1].m[j] : ax.E[1].m[j];
@@ -398,7 +398,7 @@ struct SpeciesTarget {
       }
       t = cE * Em - gE * ek;
     }
-    return (t - gd * dl) + qY * sum;
+    return t;
   }
 };
 
@@ -410,9 +410,9 @@ struct Mixture {
   R Dq[D];                   // half of (omega - omega1)(q* - q^eq) (Eq. 54, Eq. 55)
   R U, hw2;                  // specific internal energy, w^2/2
 
+  // what does not depend on the diffusion velocities
   template <int M, bool EN>
-  LBM_HD void compute(const Params<R>& p, const Moments<R, D, M, EN, true>& mo, const State<R, D, M>& s, R inv_phi,
-                      const Transport<R, D, M>& tr, const Grad<R, D, M, EN>& gr) {
+  LBM_HD void scalars(const Params<R>& p, const State<R, D, M>& s, R inv_phi, R divu) {
     // Eq. 65, Eq. 67: 1/omega = 1/2 + mu/P, P of Eq. 3
     RT = s.Rg * s.T;
     R mu = R(0);
@@ -423,14 +423,19 @@ struct Mixture {
     inv_om = R(0.5) + muP;
     omega = R(1) / inv_om;
     omega1 = R(1) / (R(0.5) + muP * p.inv_Pr);
-    bdu = mu * (R(2) / R(D) - p.bulk_ratio - (EN ? s.Rg * s.inv_cv : R(0))) * gr.divu;
+    bdu = mu * (R(2) / R(D) - p.bulk_ratio - (EN ? s.Rg * s.inv_cv : R(0))) * divu;
+  }
+
+  // Knudsen force (part of the momentum lattice) and the mass average of v
+  template <int M>
+  LBM_HD void force(const State<R, D, M>& s, const R* inv_tauk, const R (*v)[D], R* vbar) {
     // component velocity u* + (V_a - Vbar): diffusion velocities taken
     // relative to the species' mass average, the mixture velocity at the
     // middle of the step (trapezoidal drag of the mixture; reading R8)
-    R ks[M], kdrag = R(0), vbar[D];
+    R ks[M], kdrag = R(0);
 #pragma unroll
     for (int a = 0; a < M; ++a) {
-      ks[a] = s.sa[a] * tr.inv_tauk[a];
+      ks[a] = s.sa[a] * inv_tauk[a];
       kdrag += ks[a];
     }
     const R drag = R(1) / (R(1) + R(0.5) * kdrag * s.inv_sf);
@@ -438,12 +443,18 @@ struct Mixture {
     for (int b = 0; b < D; ++b) {
       vbar[b] = R(0);
 #pragma unroll
-      for (int a = 0; a < M; ++a) vbar[b] += s.Y[a] * tr.v[a][b];
+      for (int a = 0; a < M; ++a) vbar[b] += s.Y[a] * v[a][b];
       R f = kdrag * (s.w[b] - vbar[b]);
 #pragma unroll
-      for (int a = 0; a < M; ++a) f += ks[a] * tr.v[a][b];
+      for (int a = 0; a < M; ++a) f += ks[a] * v[a][b];
       Fk[b] = -drag * f;
     }
+  }
+
+  // first-order part of the energy lattice (Eq. 54, Eq. 55)
+  template <int M, bool EN>
+  LBM_HD void heat(const Params<R>& p, const Moments<R, D, M, EN, true>& mo, const State<R, D, M>& s, const R (*v)[D],
+                   const R* vbar, const Grad<R, D, M, EN>& gr) {
     U = R(0);
     hw2 = R(0);
     if (EN) {
@@ -468,7 +479,7 @@ struct Mixture {
         R sV = -HYs * vbar[b], sdY = R(0);
 #pragma unroll
         for (int a = 0; a < M; ++a) {
-          sV += HY[a] * tr.v[a][b];
+          sV += HY[a] * v[a][b];
           sdY += Ha[a] * gr.dY[a][b];
         }
         const R d = dom * (mo.q[b] - uP - (s.E + RT) * s.jf[b]) + omega1 * s.sf * sV +
@@ -476,6 +487,15 @@ struct Mixture {
         Dq[b] = R(0.5) * d;
       }
     }
+  }
+
+  template <int M, bool EN>
+  LBM_HD void compute(const Params<R>& p, const Moments<R, D, M, EN, true>& mo, const State<R, D, M>& s, R inv_phi,
+                      const Transport<R, D, M>& tr, const Grad<R, D, M, EN>& gr) {
+    R vbar[D];
+    scalars<M, EN>(p, s, inv_phi, gr.divu);
+    force<M>(s, tr.inv_tauk, tr.v, vbar);
+    heat<M, EN>(p, mo, s, tr.v, vbar, gr);
   }
 
   // axis moments of the extended equilibrium (Eq. 44, Eq. 45; reading of u^ex)
@@ -541,19 +561,15 @@ LBM_HD bool bad_state(const State<R, D, M>& s, R inv_phi) {
 
 // Collision and store of one D2Q9 node given its streamed populations
 // (through the puller), its moments, state and gradient inputs (a4-a9).
-// With COEF, coef[l] receives the derivative of every non-rest post-collision
-// population of lattice l with respect to its own streamed population at
-// fixed moments (1 - 2 beta_a for the species, 1 - omega for the momentum and
-// energy lattices): the adjoint needs it, the step does not.
-template <class R, int D, int M, bool EN, class PullF, bool COEF = false>
+template <class R, int D, int M, bool EN, class PullF>
 LBM_HD void collide_gen(const Params<R>& p, const PullF& pf, int n, const Moments<R, D, M, EN, true>& mo,
-                        const State<R, D, M>& s, const Grad<R, D, M, EN>& gr, R* __restrict__ dst, int* status,
-                        R* coef = nullptr) {
+                        const State<R, D, M>& s, const Grad<R, D, M, EN>& gr, R* __restrict__ dst, int* status) {
   static_assert(D == 2, "D3Q27 nodes collide lattice by lattice (lbm_split3d.cuh)");
   constexpr int Q = Lat<D>::Q;
   constexpr int REST = (Q - 1) / 2;
   const unsigned N = (unsigned)p.N;
   R* __restrict__ dn = dst + n;
+  auto put = [&](int l, int i, const R& v) { dn[(size_t)(unsigned)(l * Q + i) * N] = v; };
   const R inv_phi = R(1) / s.phi;
   if (bad_state(s, inv_phi)) flag(status, 1);
 
@@ -562,12 +578,6 @@ LBM_HD void collide_gen(const Params<R>& p, const PullF& pf, int n, const Moment
   if (tr.used_fp64) flag(status, 2);
   Mixture<R, D> mix;
   mix.template compute<M, EN>(p, mo, s, inv_phi, tr, gr);
-  if constexpr (COEF) {
-#pragma unroll
-    for (int a = 0; a < M; ++a) coef[a] = R(1) - R(2) * tr.beta[a];
-    coef[M] = R(1) - mix.omega;
-    if (EN) coef[M + 1] = R(1) - mix.omega;
-  }
 
   // ---- species (Eq. 21, Eq. 25) --------------------------------------------
   {
@@ -581,31 +591,21 @@ LBM_HD void collide_gen(const Params<R>& p, const PullF& pf, int n, const Moment
 #pragma unroll
     for (int a = 0; a < M; ++a) {
       SpeciesTarget<R, D> t;
+      const R gd = tr.q[a] * tr.inv_tauk[a], qY = tr.q[a] * s.Y[a] * tr.C;
       t.cE = R(2) * tr.beta[a] * s.sa[a];
-      t.gd = tr.q[a] * tr.inv_tauk[a];
-      t.gE = t.gd * s.sa[a];
-      t.qY = tr.q[a] * s.Y[a] * tr.C;
+      t.gE = gd * s.sa[a];
       t.th = R(0.5) * p.Ra[a] * s.T;
-      R T[9];
+      R X[M], T[9];
 #pragma unroll
-      for (int j = 0; j < 3; ++j)
+      for (int b = 0; b < M; ++b) X[b] = (b == a) ? -gd : qY * p.invDmm[a][b];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          const int e = i + 3 * j;
-          if (e == 0) continue;
-          R sum = R(0);
-          bool first = true;
+      for (int e = 1; e < 9; ++e) {
+        T[e] = t.template entry<0>(ax[a], s.w, e % 3, e / 3);
 #pragma unroll
-          for (int b = 0; b < M; ++b)
-            if (b != a) {
-              if (first) sum = p.invDmm[a][b] * dl[b][e];
-              else sum += p.invDmm[a][b] * dl[b][e];
-              first = false;
-            }
-          T[e] = t.template entry<0>(ax[a], s.w, i, j, dl[a][e], sum);
-        }
-      const R acc = relax_slice<R, D, false>(pf, a, 0, R(1) - R(2) * tr.beta[a], T, nullptr, dn, N);
-      dn[(size_t)(unsigned)(a * Q + REST) * N] = mo.sa[a] - acc;
+        for (int b = 0; b < M; ++b) T[e] += X[b] * dl[b][e];
+      }
+      const R acc = relax_slice<R, D, false>(pf, a, R(1) - R(2) * tr.beta[a], T, nullptr, put);
+      put(a, REST, mo.sa[a] - acc);
     }
   }
   const R keep = R(1) - mix.omega;
@@ -616,15 +616,15 @@ LBM_HD void collide_gen(const Params<R>& p, const PullF& pf, int n, const Moment
     for (int b = 0; b < D; ++b) mix.momentum_axis(s.w[b], s.inv_sf, b, gr.dPi[b], F[b]);
     R m[1][9];
     product_moments<R, D>(mix.omega * s.sf, F, m);
-    const R acc = relax_slice<R, D, false>(pf, M, 0, keep, m[0], nullptr, dn, N);
-    dn[(size_t)(unsigned)(M * Q + REST) * N] = mo.sf - acc;
+    const R acc = relax_slice<R, D, false>(pf, M, keep, m[0], nullptr, put);
+    put(M, REST, mo.sf - acc);
   }
   // ---- energy (Eq. 43, Eq. 51, Eq. 54) ------------------------------------------
   if (EN) {
     R m[1][9];
     energy_moments<R, D>(mix.omega * s.sf * mix.U, mix.omega * s.sf, mix.RT, s.w, m);
-    const R acc = relax_slice<R, D, true>(pf, M + 1, 0, keep, m[0], mix.Dq, dn, N);
-    dn[(size_t)(unsigned)((M + 1) * Q + REST) * N] = mo.sg - acc;
+    const R acc = relax_slice<R, D, true>(pf, M + 1, keep, m[0], mix.Dq, put);
+    put(M + 1, REST, mo.sg - acc);
   }
 }
 

@@ -33,30 +33,31 @@ struct Launch {
   template <bool AUX>
   static int macro3(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, R* aux, cudaStream_t s) {
     if constexpr (D == 3) {
-      constexpr size_t smem = split_smem_bytes<R, M, EN>(NB, false);
+      constexpr size_t smem = split_smem_bytes<R, M, EN>(NB, false, false);
       k_macro3<R, M, EN, NB, AUX><<<(p.N + NB - 1) / NB, NB * L, smem, s>>>(p, it, a, aux);
     }
     return 0;
   }
-  template <bool SRC, int MINB>
+  template <bool SRC, int MINB, bool PARK>
   static int collide3(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, const double* src,
                       cudaStream_t s) {
     if constexpr (D == 3) {
-      constexpr size_t smem = split_smem_bytes<R, M, EN>(NB, true);
-      auto kern = k_collide3<R, M, EN, NB, SRC, MINB>;
+      constexpr size_t smem = split_smem_bytes<R, M, EN>(NB, true, PARK);
+      auto kern = k_collide3<R, M, EN, NB, SRC, MINB, PARK>;
       static bool done = false;
       if (configure(kern, smem, done)) return -1;
       kern<<<(p.N + NB - 1) / NB, NB * L, smem, s>>>(p, it, a, src);
     }
     return 0;
   }
-  static constexpr int kMinB = sizeof(R) == 4 ? 2 : 1;
+  static constexpr int kMinB = 2;
+  static constexpr bool kPark = sizeof(R) == 4;
   static void macro(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
     if constexpr (D == 3) macro3<false>(p, it, a, nullptr, s);
     else k_macro<R, D, M, EN><<<grid(p.N), block(p.N), 0, s>>>(p, it, a);
   }
   static void collide(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
-    if constexpr (D == 3) collide3<false, kMinB>(p, it, a, nullptr, s);
+    if constexpr (D == 3) collide3<false, kMinB, kPark>(p, it, a, nullptr, s);
     else k_collide<R, D, M, EN><<<grid(p.N), block(p.N), 0, s>>>(p, it, a);
   }
   // fused step, shared-memory halo ring, tile TX x TY marching SEG planes
@@ -164,12 +165,12 @@ struct Launch {
     } else {
       macro3<false>(p, it, a, nullptr, s);
       switch (v) {
-        case 0: return collide3<false, 1>(p, it, a, nullptr, s);
-        case 1: return collide3<false, 2>(p, it, a, nullptr, s);
-        case 2: return collide3<false, sizeof(R) == 4 ? 3 : 1>(p, it, a, nullptr, s);
-        case 3: return collide3<false, sizeof(R) == 4 ? 4 : 1>(p, it, a, nullptr, s);
-        case 4: return collide3<false, kMinB>(p, it, a, nullptr, s);
-        case 5: return collide3<false, kMinB>(p, it, a, nullptr, s);
+        case 0: return collide3<false, 1, false>(p, it, a, nullptr, s);
+        case 1: return collide3<false, 2, false>(p, it, a, nullptr, s);
+        case 2: return collide3<false, sizeof(R) == 4 ? 3 : 2, false>(p, it, a, nullptr, s);
+        case 3:
+        case 4:
+        case 5: return collide3<false, kMinB, kPark>(p, it, a, nullptr, s);
         default: return -1;
       }
     }
@@ -200,7 +201,7 @@ struct Launch {
   }
   static void react_collide(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, const ReactArgs& ra,
                             cudaStream_t s) {
-    if constexpr (has_react) collide3<true, kMinB>(p, it, a, ra.src, s);
+    if constexpr (has_react) collide3<true, kMinB, kPark>(p, it, a, ra.src, s);
   }
   static Ops<R> ops() {
     return Ops<R>{macro, collide, fused, n_variants, init, moments, has_react ? react_macro : nullptr,

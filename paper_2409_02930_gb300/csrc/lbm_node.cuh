@@ -167,7 +167,7 @@ struct Transport {
       const R isa = R(1) / s.sa[a];
 #pragma unroll
       for (int b = 0; b < D; ++b)
-        B[a][b] = (tiny ? R(0) : (ja[a * D + b] * isa - s.w[b])) - hk * s.w[b];
+        B[a][b] = (tiny ? R(0) : ja[a * D + b] * isa - s.w[b]) - hk * s.w[b];
     }
     used_fp64 = 0;
     if constexpr (std::is_same<R, float>::value) {
@@ -191,8 +191,11 @@ struct Transport {
   // non-equilibrium populations), FP32 leaves j_a / rho_a to rounding noise,
   // which the quasi-equilibrium then amplifies.
   LBM_HD static bool unresolved(const State<R, D, M>& s, const R* sabs, int a) {
-    bool tiny = s.sa[a] < R(1e-14) * s.ss;
-    if (ScalarTraits<R>::single) tiny = tiny || !(sabs[a] <= R(1e4) * s.sa[a]);
+    return unresolved(s.sa[a], s.ss, sabs[a]);
+  }
+  LBM_HD static bool unresolved(R sa, R ss, R sabs) {
+    bool tiny = sa < R(1e-14) * ss;
+    if (ScalarTraits<R>::single) tiny = tiny || !(sabs <= R(1e4) * sa);
     return tiny;
   }
 

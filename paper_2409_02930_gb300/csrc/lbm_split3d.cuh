@@ -5,95 +5,241 @@
 //
 // What bounds it.  With a thread per node, 216 staged populations (55 KB of
 // shared memory per 64 threads) and 255 registers left 8 warps per SM and
-// straight-line code of 14,000 instructions per node: at 64 x 32 x 32 (FP32)
-// the node update took 91.8 us at 32 % issue, its first pass 56.6 us at 21 %.
-// Split by lattice a thread needs about 100 registers and the block's groups
-// run the same short code for their own species.
+// straight-line code of 14,000 instructions per node: 5.6 ms per step of the
+// 256 x 128 x 128 FP32 anode.  Split by lattice the block's groups run the same
+// short code for their own species.  Whatever one group did alone for the
+// whole block then set its pace (instructions that one warp runs once are
+// fetched at about eight cycles each: state and transport of the 32 nodes in
+// the last group 5,700 cycles, six derivatives in the momentum group 7,600, of
+// 14,000 in all), so the species' groups now share that work too.
 //
 // The first pass (k_macro3) sums every lattice and lets one group form the
-// macro fields.  The node update (k_collide3) pulls again, takes its gradient
-// inputs directly from the neighbours' macro fields (group a differentiates
-// Y_a, the last two groups u and Pi; they hit L1/L2, which is cheaper than a
-// pass that writes and re-reads 22 fields), forms state, transport and
-// mixture quantities once per node in one group, shares the species'
-// difference moments d_b (26 per species) through shared memory for the
-// coupling sum of Eq. 25, and relaxes each lattice in its own group.
+// macro fields.  In the node update (k_collide3)
+//   - every species' group pulls, sums, differentiates its Y_a and one of u and
+//     Pi straight from the neighbours' macro fields (they hit L1/L2; a pass of
+//     its own wrote and re-read 22 fields);
+//   - the last group forms the state; the species' groups set up their row of
+//     the diffusion system and solve it together (Gauss-Jordan, the pivot row
+//     through shared memory; the matrix is row diagonally dominant);
+//   - the species share their difference moments d_b (26 each) through shared
+//     memory for the coupling sum of Eq. 25, read 16 bytes at a time and summed
+//     two at a time (packed FP32 multiply-add), while the last group forms the
+//     mixture quantities; every group relaxes its own lattice.
 #pragma once
 
 #include "lbm_surface.cuh"
 
 namespace lbm {
 
-// Fields of a node in shared memory, [field][NB].
-template <int M, bool EN>
+// Fields of a node in shared memory, [field][NB], then the species'
+// difference moments [M][NB][kStride]: z order 0 at kO0 (8 entries, without
+// the zeroth moment), 1 at kO1 and 2 at kO2 (9 each).  The stride is an odd
+// number of 16-byte units, so 16-byte accesses of consecutive nodes touch
+// every bank once.
+template <class R, int M, bool EN>
 struct SplitFields {
   // sums: per species sa, j, sum |f|; momentum sf, j, Pt (6); energy sg, q
   static constexpr int kSp = 5, kMo = kSp * M, kEn = kMo + 10, kSums = kEn + (EN ? 4 : 0);
-  // gradient inputs
-  static constexpr int kDiv = kSums, kPi = kDiv + 1, kDY = kPi + 3, kGrad = kDY + (EN ? 3 * M : 0);
-  // node quantities: per species v, sa, beta, gd, qY, source; then the mixture's
-  static constexpr int kCo = kGrad, kCoN = 8, kMix = kCo + kCoN * M;
-  static constexpr int kW = kMix, kT = kW + 3, kF = kT + 1 /* xi, Pex */, kOm = kF + 6, kCf = kOm + 1,
-                       kRt = kCf + 1, kCu = kRt + 1, kC2 = kCu + 1, kDq = kC2 + 1, kTot = kDq + 3 /* sf, sg */,
-                       kEnd = kTot + 2;
-  // the species' difference moments (26 each) reuse the sums' and gradients' place
-  static constexpr int kDelta = kEnd;
-  static constexpr int kAll = kDelta + 26 * M;
+  // gradient inputs: d_b u_b, d_b Pi_b, d_b Y_a
+  static constexpr int kU = kSums, kDY = kU + 6, kGrad = kDY + (EN ? 3 * M : 0);
+  // state: w, T, sum of sa, sqrt(T)/phi, Y_b C/2; row sums and margins of the
+  // diffusion system; v_a; sources
+  static constexpr int kW = kGrad, kT = kW + 3, kSS = kT + 1, kKT = kSS + 1, kHY = kKT + 1, kCond = kHY + M,
+                       kV = kCond + 2 * M, kRd = kV + 3 * M;
+  // momentum axes, relaxation, prefactor, total; pivot rows
+  static constexpr int kF = kRd + M, kOm = kF + 6, kCf = kOm + 1, kTot = kCf + 1, kPv = kTot + 1,
+                       kAll = kPv + M * (M + 3);
+  static constexpr int kStride = sizeof(R) == 4 ? 36 : 30, kO0 = 0, kO1 = 8, kO2 = sizeof(R) == 4 ? 20 : 18;
 };
 
+// With PARK the populations wait in shared memory, not in registers, between
+// their sums and their relaxation.
 template <class R, int M, bool EN>
-constexpr size_t split_smem_bytes(int NB, bool collide) {
-  using F = SplitFields<M, EN>;
-  return sizeof(R) * (size_t)NB * (collide ? F::kAll : F::kSums);
+constexpr size_t split_smem_bytes(int NB, bool collide, bool park) {
+  using F = SplitFields<R, M, EN>;
+  return sizeof(R) * (size_t)NB *
+         (collide ? F::kAll + M * F::kStride + (park ? 27 * (M + 1 + (EN ? 1 : 0)) : 0) : F::kSums);
 }
 
-// Pulls lattice l of node (x, y, z).
+// lattice of this thread's warp, known to the compiler as one value per warp
+// (addresses of the lattice's planes then come from uniform registers)
+template <int NB>
+__device__ __forceinline__ int group_of() {
+  static_assert(NB % 32 == 0, "a warp holds one lattice");
+  return __shfl_sync(0xffffffffu, (int)threadIdx.x / NB, 0);
+}
+
+// named barriers among `n` threads of the block
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(n) : "memory"); }
+
+// two values as one register pair: FP32 pairs use the packed multiply-add
+template <class R> struct Pair;
+template <> struct Pair<float> {
+  unsigned long long v;
+  __device__ __forceinline__ static Pair make(float a, float b) {
+    Pair p;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(p.v) : "f"(a), "f"(b));
+    return p;
+  }
+  __device__ __forceinline__ void fma(const Pair& a, const Pair& b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v) : "l"(a.v), "l"(b.v));
+  }
+  __device__ __forceinline__ void get(float& a, float& b) const { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+};
+template <> struct Pair<double> {
+  double a, b;
+  __device__ __forceinline__ static Pair make(double x, double y) { return Pair{x, y}; }
+  __device__ __forceinline__ void fma(const Pair& x, const Pair& y) {
+    a += x.a * y.a;
+    b += x.b * y.b;
+  }
+  __device__ __forceinline__ void get(double& x, double& y) const {
+    x = a;
+    y = b;
+  }
+};
+// 16 bytes of shared memory as pairs
+__device__ __forceinline__ void load16(const float* s, Pair<float>* o) {
+  const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(s);
+  o[0].v = t.x;
+  o[1].v = t.y;
+}
+__device__ __forceinline__ void load16(const double* s, Pair<double>* o) {
+  const double2 t = *reinterpret_cast<const double2*>(s);
+  o[0] = Pair<double>{t.x, t.y};
+}
+
+// CNT values to shared memory, 16 bytes at a time (the last unit padded)
+template <int CNT>
+__device__ __forceinline__ void store16(float* s, const float* m) {
+#pragma unroll
+  for (int q = 0; q < CNT; q += 4)
+    *reinterpret_cast<float4*>(s + q) = make_float4(m[q], q + 1 < CNT ? m[q + 1] : 0.f, q + 2 < CNT ? m[q + 2] : 0.f,
+                                                    q + 3 < CNT ? m[q + 3] : 0.f);
+}
+template <int CNT>
+__device__ __forceinline__ void store16(double* s, const double* m) {
+#pragma unroll
+  for (int q = 0; q < CNT; q += 2)
+    *reinterpret_cast<double2*>(s + q) = make_double2(m[q], q + 1 < CNT ? m[q + 1] : 0.0);
+}
+
+// sum_b X[b] d_b of CNT difference moments at offset OFF: 16 bytes per read
+template <class R, int M, int STRIDE, int NB, int CNT>
+__device__ __forceinline__ void couple(const R* __restrict__ d, const R (&X)[M], R (&out)[9]) {
+  constexpr int PER = 16 / (int)sizeof(R), NV = (CNT + PER - 1) / PER, NP = NV * PER / 2;
+  Pair<R> acc[NP];
+#pragma unroll
+  for (int q = 0; q < NP; ++q) acc[q] = Pair<R>::make(R(0), R(0));
+#pragma unroll
+  for (int b = 0; b < M; ++b) {
+    const Pair<R> x = Pair<R>::make(X[b], X[b]);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      Pair<R> v[PER / 2];
+      load16(d + b * NB * STRIDE + q * PER, v);
+#pragma unroll
+      for (int k = 0; k < PER / 2; ++k) acc[q * (PER / 2) + k].fma(x, v[k]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < NP; ++q) {
+    R a, b;
+    acc[q].get(a, b);
+    if (2 * q < CNT) out[2 * q] = a;
+    if (2 * q + 1 < CNT) out[2 * q + 1] = b;
+  }
+}
+
+// Row offsets (elements) of the 3 x 3 neighbouring rows of node (x, y, z) and
+// the x offsets of its neighbours (wrapped, or clamped to the boundary node
+// with CLAMP at open faces).
+template <class R>
+struct Rows3 {
+  int row[3][3];          // [z + cz][y + cy] rows, at column x
+  int dx[3];
+  template <bool CLAMP>
+  __device__ __forceinline__ void init(const Params<R>& p, int x, int y, int z) {
+    const int ys[3] = {wrapi(y - 1, p.ny), y, wrapi(y + 1, p.ny)}, zs[3] = {wrapi(z - 1, p.nz), z, wrapi(z + 1, p.nz)};
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) row[c][b] = x + p.nx * (ys[b] + p.ny * zs[c]);
+    dx[0] = x > 0 ? -1 : ((CLAMP && p.bc_lo != BC_PERIODIC) ? 0 : p.nx - 1);
+    dx[1] = 0;
+    dx[2] = x < p.nx - 1 ? 1 : ((CLAMP && p.bc_hi != BC_PERIODIC) ? 0 : 1 - p.nx);
+  }
+};
+
+// Velocity of the reservoir ghost beside face node (x, y, z) (the adjacent
+// node's, all of whose sources are inside); rolled loops, few nodes take it.
+template <class R, int M>
+__device__ __forceinline__ void ghost_velocity3(const Params<R>& p, const R* __restrict__ src,
+                                                const R* __restrict__ phiA, int x, int y, int z, Ghost<R, 3>& gh) {
+  gh.side = x == 0 ? 0 : 1;
+  const int xa = gh.side == 0 ? 1 : p.nx - 2;
+  R s0 = R(0), jx = R(0), jy = R(0), jz = R(0);
+#pragma unroll 1
+  for (int cz = -1; cz <= 1; ++cz)
+#pragma unroll 1
+    for (int cy = -1; cy <= 1; ++cy) {
+      const R* q = src + (size_t)(unsigned)(M * 27 + 3 * (cy + 1) + 9 * (cz + 1)) * (unsigned)p.N +
+                   (xa + p.nx * (wrapi(y - cy, p.ny) + p.ny * wrapi(z - cz, p.nz)));
+      const R a = q[1], b = q[(size_t)(unsigned)p.N], c = q[(size_t)2 * (unsigned)p.N - 1];
+      const R r = a + c + b;
+      s0 += r;
+      jx += c - a;
+      jy += R(cy) * r;
+      jz += R(cz) * r;
+    }
+  const R rho_f = s0 / phiA[xa + p.nx * (y + p.ny * z)];
+  gh.u[0] = jx / rho_f;
+  gh.u[1] = jy / rho_f;
+  gh.u[2] = jz / rho_f;
+  gh.phi = phiA[x + p.nx * (y + p.ny * z)];
+}
+
+// Pulls lattice l of node (x, y, z).  Every address is a row pointer plus the
+// direction's plane (one wide multiply-add each); the planes' byte stride fits
+// 32 bits because a D3Q27 state that fits the card has fewer than 2^29 nodes.
+// Open faces load their wrapped column first and are patched below.
 template <class R, int M, bool EN>
 __device__ __forceinline__ void pull_lattice(const Params<R>& p, const InletTables<R>& it, const R* __restrict__ src,
                                              const R* __restrict__ phiA, int x, int y, int z, int l, R (&f)[27]) {
-  const unsigned N = (unsigned)p.N;
-  const R* __restrict__ fl = src + (size_t)(unsigned)(l * 27) * N;
-  const int n = x + p.nx * (y + p.ny * z);
-  // columns of the three x shifts; open faces read their own node (bounce-back
-  // swaps the direction, reservoir values are overwritten below)
-  int xs[3];
-  bool open[3] = {false, false, false};
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const int s = x - (c - 1);
-    xs[c] = s;
-    if (s < 0 || s >= p.nx) {
-      open[c] = (s < 0 ? p.bc_lo : p.bc_hi) != BC_PERIODIC;
-      xs[c] = wrapi(s, p.nx);
-    }
-  }
-  const int ys[3] = {wrapi(y + 1, p.ny), y, wrapi(y - 1, p.ny)}, zs[3] = {wrapi(z + 1, p.nz), z, wrapi(z - 1, p.nz)};
+  const unsigned plane = (unsigned)p.N * (unsigned)sizeof(R);
+  const char* fl = reinterpret_cast<const char*>(src) + (size_t)(unsigned)(l * 27) * plane;
+  Rows3<R> r;
+  r.template init<false>(p, x, y, z);
 #pragma unroll
   for (int cz = 0; cz < 3; ++cz)
 #pragma unroll
-    for (int cy = 0; cy < 3; ++cy) {
-      const int row = p.nx * (ys[cy] + p.ny * zs[cz]);
+    for (int cy = 0; cy < 3; ++cy)
 #pragma unroll
       for (int cx = 0; cx < 3; ++cx) {
         const int i = cx + 3 * cy + 9 * cz;
-        int s = row + xs[cx];
-        unsigned ii = i;
-        if (cx != 1 && open[cx]) {
-          s = n;
-          ii = 26 - i;
-        }
-        f[i] = fl[(size_t)ii * N + s];
+        const R* q = reinterpret_cast<const R*>(fl + (size_t)(unsigned)i * plane);
+        f[i] = q[r.row[2 - cz][2 - cy] + r.dx[2 - cx]];
       }
+  const bool flo = x == 0 && p.bc_lo != BC_PERIODIC, fhi = x == p.nx - 1 && p.bc_hi != BC_PERIODIC;
+  if (flo || fhi) {
+    const int n = r.row[1][1];
+    if ((flo ? p.bc_lo : p.bc_hi) == BC_BOUNCEBACK) {
+#pragma unroll
+      for (int i = 0; i < 27; i += 3) {
+        const R v = reinterpret_cast<const R*>(fl + (size_t)(unsigned)(flo ? 24 - i : 26 - i) * plane)[n];
+        if (flo) f[i + 2] = v;
+        else f[i] = v;
+      }
+    } else {
+      Ghost<R, 3> gh;
+      ghost_velocity3<R, M>(p, src, phiA, x, y, z, gh);
+      ghost_lattice<R, 3, M, EN>(p, it, gh, l, [&](int cy, int cz, const R& v) {
+        const int row = 1 + 3 * (cy + 1) + 9 * (cz + 1);
+        if (flo) f[row + 1] = v;
+        else f[row - 1] = v;
+      });
     }
-  const bool lo = x == 0 && p.bc_lo == BC_INLET, hi = x == p.nx - 1 && p.bc_hi == BC_INLET;
-  if (lo || hi) {
-    Ghost<R, 3> gh;
-    ghost_velocity<R, 3, M>(p, src, phiA, x, y, z, gh);
-    ghost_lattice<R, 3, M, EN>(p, it, gh, l, [&](int cy, int cz, const R& v) {
-      const int row = 1 + 3 * (cy + 1) + 9 * (cz + 1);
-      if (lo) f[row + 1] = v;
-      else f[row - 1] = v;
-    });
   }
 }
 
@@ -102,25 +248,24 @@ __device__ __forceinline__ void pull_lattice(const Params<R>& p, const InletTabl
 template <class R, int M, bool EN, int NB, bool AUX>
 __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0))) k_macro3(Params<R> p, InletTables<R> it, StepArgs<R> a,
                                                                        R* __restrict__ aux) {
-  using F = SplitFields<M, EN>;
-  extern __shared__ unsigned char smem_raw[];
-  const int lane = threadIdx.x % NB, l = threadIdx.x / NB;
+  using F = SplitFields<R, M, EN>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x % NB, l = group_of<NB>();
   R* S = reinterpret_cast<R*>(smem_raw) + lane;
   const int n = min((int)(blockIdx.x * NB) + lane, p.N - 1);
-  int x, y, z;
-  node_xyz<R, 3>(p, n, x, y, z);
-  R f[27];
-  pull_lattice<R, M, EN>(p, it, a.src, a.phi, x, y, z, l, f);
-  auto get = [&](int i) { return f[i]; };
-  R s, j[3], Pt[3][3];
-  if (l == M) {
-    lattice_sums<R, 3, 1>(get, s, j, Pt);
-    S[F::kMo * NB] = s;
+  {
+    int x, y, z;
+    node_xyz<R, 3>(p, n, x, y, z);
+    R f[27];
+    pull_lattice<R, M, EN>(p, it, a.src, a.phi, x, y, z, l, f);
+    // every group takes the first moments: one code path for all lattices
+    R s, j[3], Pt[3][3];
+    lattice_sums<R, 3, 1>([&](int i) { return f[i]; }, s, j, Pt);
+    S[(l < M ? F::kSp * l : (l == M ? F::kMo : F::kEn)) * NB] = s;
+    if (l == M) {
 #pragma unroll
-    for (int b = 0; b < 3; ++b) S[(F::kMo + 1 + b) * NB] = j[b];
-  } else {
-    lattice_sums<R, 3, 0>(get, s, j, Pt);
-    S[(l < M ? F::kSp * l : F::kEn) * NB] = s;
+      for (int b = 0; b < 3; ++b) S[(F::kMo + 1 + b) * NB] = j[b];
+    }
   }
   __syncthreads();
   if (l != 0 || (int)(blockIdx.x * NB) + lane >= p.N) return;
@@ -141,221 +286,148 @@ __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0))) k_macro3(Params<R
   }
 }
 
-// Isotropic derivatives of one macro field at a node, from its 27-point
-// neighbourhood (zero-gradient copy across open x faces): smoothing weights
-// (1/6, 2/3, 1/6) along the other axes, central difference along the axis.
+// Isotropic derivatives of macro field g at a node from its 27-point
+// neighbourhood: smoothing weights (1/6, 2/3, 1/6) along the other axes,
+// central difference along the axis.
 template <class R>
-struct Stencil3 {
-  unsigned row[3][3];
-  int xs[3];
-  __device__ __forceinline__ void init(const Params<R>& p, int x, int y, int z) {
+__device__ __forceinline__ void grad3(const Rows3<R>& r, const R* __restrict__ g, R (&o)[3]) {
+  const R w0 = R(2) / R(3), w1 = R(1) / R(6);
+  R sx[3][3], t[3];
+  o[0] = R(0);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      int s = x + c - 1;
-      if (s < 0) s = (p.bc_lo == BC_PERIODIC) ? s + p.nx : 0;
-      if (s >= p.nx) s = (p.bc_hi == BC_PERIODIC) ? s - p.nx : p.nx - 1;
-      xs[c] = s;
+  for (int c = 0; c < 3; ++c) {
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const R* q = g + r.row[c][b];
+      const R lo = q[r.dx[0]], hi = q[r.dx[2]];
+      const R w = R(0.5) * (b == 1 ? w0 : w1) * (c == 1 ? w0 : w1);
+      o[0] += w * (hi - lo);
+      sx[c][b] = w1 * (lo + hi) + w0 * q[0];
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int b = 0; b < 3; ++b)
-        row[c][b] = (unsigned)(p.nx * (wrapi(y + b - 1, p.ny) + p.ny * wrapi(z + c - 1, p.nz)));
+    t[c] = sx[c][2] - sx[c][0];
   }
-  template <bool DX, bool DY, bool DZ>
-  __device__ __forceinline__ void grad(const R* __restrict__ g, R& gx, R& gy, R& gz) const {
-    const R w0 = R(2) / R(3), w1 = R(1) / R(6);
-    R sx[3][3], dx[3][3];
+  o[1] = R(0.5) * (w1 * (t[0] + t[2]) + w0 * t[1]);
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
+  for (int b = 0; b < 3; ++b) t[b] = sx[2][b] - sx[0][b];
+  o[2] = R(0.5) * (w1 * (t[0] + t[2]) + w0 * t[1]);
+}
+
+// Derivative of field g along `axis` (0 x, 1 y, 2 z) only.
+template <class R>
+__device__ __forceinline__ R grad_axis3(const Rows3<R>& r, const R* __restrict__ g, int axis) {
+  const R w0 = R(2) / R(3), w1 = R(1) / R(6);
+  R s = R(0);
 #pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        if (!DX && ((!DY && c == 1) || (!DZ && b == 1))) continue;
-        const R* q = g + row[c][b];
-        const R lo = q[xs[0]], hi = q[xs[2]];
-        if (DX) dx[c][b] = hi - lo;
-        if (DY || DZ) sx[c][b] = w1 * (lo + hi) + w0 * q[xs[1]];
-      }
-    if (DX) {
-      R t[3];
+  for (int c = 0; c < 3; ++c)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) t[c] = w1 * (dx[c][0] + dx[c][2]) + w0 * dx[c][1];
-      gx = R(0.5) * (w1 * (t[0] + t[2]) + w0 * t[1]);
+    for (int b = 0; b < 3; ++b) {
+      // c, b run over the other two axes; the pair along the axis is lo, hi
+      const R w = R(0.5) * (b == 1 ? w0 : w1) * (c == 1 ? w0 : w1);
+      const int lo = axis == 0 ? r.row[c][b] + r.dx[0] : (axis == 1 ? r.row[c][0] + r.dx[b] : r.row[0][c] + r.dx[b]);
+      const int hi = axis == 0 ? r.row[c][b] + r.dx[2] : (axis == 1 ? r.row[c][2] + r.dx[b] : r.row[2][c] + r.dx[b]);
+      s += w * (g[hi] - g[lo]);
     }
-    if (DY) {
-      R t[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) t[c] = sx[c][2] - sx[c][0];
-      gy = R(0.5) * (w1 * (t[0] + t[2]) + w0 * t[1]);
-    }
-    if (DZ) {
-      R t[3];
-#pragma unroll
-      for (int b = 0; b < 3; ++b) t[b] = sx[2][b] - sx[0][b];
-      gz = R(0.5) * (w1 * (t[0] + t[2]) + w0 * t[1]);
-    }
+  return s;
+}
+
+// Row l of the FP64 diffusion solve of one node (FP32 lattices above the
+// condition bound): the whole system from the sums in shared memory.
+template <class R, int M, bool EN, int NB>
+__device__ __noinline__ void solve_row_fp64(const Params<R>& p, const R* S, R phi, int l, R (&v)[3]) {
+  using F = SplitFields<R, M, EN>;
+  typename Transport<float, 3, M>::Fp64System y;
+  y.phi = phi; y.sf = S[F::kMo * NB]; y.T = S[F::kT * NB]; y.Kc = p.Kc;
+  const R ss = S[F::kSS * NB];
+  for (int a = 0; a < M; ++a) {
+    const R sa = S[F::kSp * a * NB];
+    y.sa[a] = sa;
+    y.Y[a] = sa / ss;
+    y.knc[a] = p.knudsen ? p.knc[a] : R(0);
+    y.tiny[a] = Transport<R, 3, M>::unresolved(sa, ss, S[(F::kSp * a + 4) * NB]);
+    for (int b = 0; b < M; ++b) y.D_[a][b] = p.invDmm[a][b];
+    for (int b = 0; b < 3; ++b) y.ja[a][b] = S[(F::kSp * a + 1 + b) * NB];
   }
-};
+  for (int b = 0; b < 3; ++b) y.w[b] = S[(F::kW + b) * NB];
+  Transport<float, 3, M>::solve_system(y);
+  for (int b = 0; b < 3; ++b) v[b] = y.v[l][b];
+}
 
 // Node update of NB nodes; with SRC the reaction sources are added: Eq. 89 to
 // the species, Eq. 87 to the momentum and Eq. 88 to the energy lattice
 // (src: [M + 2][N] in double, mass production per species, then the change of
 // the fluid internal energy).
-template <class R, int M, bool EN, int NB, bool SRC, int MINB>
+template <class R, int M, bool EN, int NB, bool SRC, int MINB, bool PARK>
 __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
     k_collide3(Params<R> p, InletTables<R> it, StepArgs<R> a, const double* __restrict__ srcv) {
-  using F = SplitFields<M, EN>;
+  using F = SplitFields<R, M, EN>;
   constexpr int L = M + 1 + (EN ? 1 : 0);
-  extern __shared__ unsigned char smem_raw[];
-  const int lane = threadIdx.x % NB, l = threadIdx.x / NB;
+  // barriers: 0 all; 1 state ready (last group to the species), 2 pivot rows
+  // (species), 3 mixture ready (last group to the momentum group), 4
+  // difference moments (species), 5 v ready (species to the last group)
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x % NB, l = group_of<NB>();
   R* S = reinterpret_cast<R*>(smem_raw) + lane;
+  R* D0 = reinterpret_cast<R*>(smem_raw) + F::kAll * NB + lane * F::kStride;
   const bool live = (int)(blockIdx.x * NB) + lane < p.N;
   const int n = live ? (int)(blockIdx.x * NB) + lane : p.N - 1;
   const unsigned N = (unsigned)p.N;
   R f[27];
+  // what the groups need after the first barrier is loaded before it, so that
+  // it waits with the pull
+  R phi = R(0), Tf = R(0), dU = R(0);
   {
     int x, y, z;
     node_xyz<R, 3>(p, n, x, y, z);
     pull_lattice<R, M, EN>(p, it, a.src, a.phi, x, y, z, l, f);
-    Stencil3<R> st;
-    st.init(p, x, y, z);
-    const R* __restrict__ mac = a.mac;
-    if (EN && l < M) {
-      R gx, gy, gz;
-      st.template grad<true, true, true>(mac + (size_t)(unsigned)(6 + l) * N, gx, gy, gz);
-      S[(F::kDY + 3 * l) * NB] = gx;
-      S[(F::kDY + 3 * l + 1) * NB] = gy;
-      S[(F::kDY + 3 * l + 2) * NB] = gz;
-    }
-    if (l == M) {
-      R gx, gy, gz, u;
-      st.template grad<true, false, false>(mac, gx, u, u);
-      st.template grad<false, true, false>(mac + N, u, gy, u);
-      st.template grad<false, false, true>(mac + (size_t)2 * N, u, u, gz);
-      S[F::kDiv * NB] = gx + gy + gz;
-    }
     if (l == L - 1) {
-      R g, u;
-      st.template grad<true, false, false>(mac + (size_t)3 * N, g, u, u);
-      S[F::kPi * NB] = g;
-      st.template grad<false, true, false>(mac + (size_t)4 * N, u, g, u);
-      S[(F::kPi + 1) * NB] = g;
-      st.template grad<false, false, true>(mac + (size_t)5 * N, u, u, g);
-      S[(F::kPi + 2) * NB] = g;
+      phi = a.phi[n];
+      if (!EN) Tf = a.Tfix[n];
+      if (SRC) dU = (R)srcv[(size_t)(unsigned)M * N + n];
     }
-  }
-  auto get = [&](int i) { return f[i]; };
-  {
-    R s, j[3], Pt[3][3];
-    if (l == M) {
-      lattice_sums<R, 3, EN ? 2 : 1>(get, s, j, Pt);
-      S[F::kMo * NB] = s;
-#pragma unroll
-      for (int b = 0; b < 3; ++b) S[(F::kMo + 1 + b) * NB] = j[b];
+    if (l < M) {
+      if (SRC) S[(F::kRd + l) * NB] = (R)srcv[(size_t)(unsigned)l * N + n];
+      Rows3<R> r;
+      r.template init<true>(p, x, y, z);
       if (EN) {
-        int k = F::kMo + 4;
+        R g[3];
+        grad3<R>(r, a.mac + (size_t)(unsigned)(6 + l) * N, g);
 #pragma unroll
-        for (int b = 0; b < 3; ++b)
-#pragma unroll
-          for (int c = b; c < 3; ++c) S[(k++) * NB] = Pt[b][c];
+        for (int b = 0; b < 3; ++b) S[(F::kDY + 3 * l + b) * NB] = g[b];
       }
-    } else {
-      lattice_sums<R, 3, 1>(get, s, j, Pt);
-      const int k = l < M ? F::kSp * l : F::kEn;
-      S[k * NB] = s;
-#pragma unroll
-      for (int b = 0; b < 3; ++b) S[(k + 1 + b) * NB] = j[b];
-      if (ScalarTraits<R>::single && l < M) {
-        R t = fabs(f[0]);
-#pragma unroll
-        for (int i = 1; i < 27; ++i) t += fabs(f[i]);
-        S[(k + 4) * NB] = t;
-      }
+#pragma unroll 1
+      for (int q = l; q < 6; q += M)
+        S[(F::kU + q) * NB] = grad_axis3<R>(r, a.mac + (size_t)(unsigned)q * N, q < 3 ? q : q - 3);
     }
   }
-  __syncthreads();
-  // ---- one group: state, transport, mixture -----------------------------------
-  if (l == L - 1) {
-    Moments<R, 3, M, EN, true> mo;
+  R* __restrict__ parked = S + (F::kAll + M * F::kStride + 27 * l) * NB;
+  auto get = [&](int i) { return PARK ? parked[i * NB] : f[i]; };
+  R s0, j0[3], sabs = R(0);
+  {
+    auto get = [&](int i) { return f[i]; };
+    R Pt[3][3];
+    const int k = l < M ? F::kSp * l : (l == M ? F::kMo : F::kEn);
+    if (EN && l == M) {
+      lattice_sums<R, 3, 2>(get, s0, j0, Pt);
+      int e = F::kMo + 4;
 #pragma unroll
-    for (int k = 0; k < M; ++k) {
-      mo.sa[k] = S[F::kSp * k * NB];
+      for (int b = 0; b < 3; ++b)
 #pragma unroll
-      for (int b = 0; b < 3; ++b) mo.ja[k][b] = S[(F::kSp * k + 1 + b) * NB];
-      if (ScalarTraits<R>::single) mo.sabs[k] = S[(F::kSp * k + 4) * NB];
+        for (int c = b; c < 3; ++c) S[(e++) * NB] = Pt[b][c];
+    } else {
+      lattice_sums<R, 3, 1>(get, s0, j0, Pt);
     }
-    mo.sf = S[F::kMo * NB];
+    S[k * NB] = s0;
 #pragma unroll
-    for (int b = 0; b < 3; ++b) mo.jf[b] = S[(F::kMo + 1 + b) * NB];
-    Grad<R, 3, M, EN> gr;
-    gr.divu = S[F::kDiv * NB];
+    for (int b = 0; b < 3; ++b) S[(k + 1 + b) * NB] = j0[b];
+    if (ScalarTraits<R>::single && l < M) {
+      sabs = fabs(f[0]);
 #pragma unroll
-    for (int b = 0; b < 3; ++b) gr.dPi[b] = S[(F::kPi + b) * NB];
-    if (EN) {
-      mo.sg = S[F::kEn * NB];
-      int k = F::kMo + 4;
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        mo.q[b] = S[(F::kEn + 1 + b) * NB];
-#pragma unroll
-        for (int c = b; c < 3; ++c) mo.Pt[b][c] = mo.Pt[c][b] = S[(k++) * NB];
-#pragma unroll
-        for (int q = 0; q < M; ++q) gr.dY[q][b] = S[(F::kDY + 3 * q + b) * NB];
-      }
+      for (int i = 1; i < 27; ++i) sabs += fabs(f[i]);
+      S[(k + 4) * NB] = sabs;
     }
-    State<R, 3, M> s;
-    s.template from_moments<EN, true>(p, mo, a.phi[n], EN ? R(0) : a.Tfix[n]);
-    const R inv_phi = R(1) / s.phi;
-    if (live && bad_state(s, inv_phi)) flag(a.status, 1);
-    Transport<R, 3, M> tr;
-    tr.compute(p, s, inv_phi, &mo.ja[0][0], mo.sabs);
-    if (live && tr.used_fp64) flag(a.status, 2);
-    R sum_rd = R(0);
+    if (PARK) {
 #pragma unroll
-    for (int k = 0; k < M; ++k) {
-      R* c = S + (F::kCo + F::kCoN * k) * NB;
-#pragma unroll
-      for (int b = 0; b < 3; ++b) c[b * NB] = tr.v[k][b];
-      c[3 * NB] = s.sa[k];
-      c[4 * NB] = tr.beta[k];
-      c[5 * NB] = tr.q[k] * tr.inv_tauk[k];
-      c[6 * NB] = tr.q[k] * s.Y[k] * tr.C;
-      if (SRC) {
-        const R rd = (R)srcv[(size_t)(unsigned)k * N + n];
-        c[7 * NB] = rd;
-        sum_rd += rd;
-      }
-    }
-    Mixture<R, 3> mix;
-    mix.template compute<M, EN>(p, mo, s, inv_phi, tr, gr);
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      Axis<R> ax;
-      mix.momentum_axis(s.w[b], s.inv_sf, b, gr.dPi[b], ax);
-      S[(F::kW + b) * NB] = s.w[b];
-      S[(F::kF + 2 * b) * NB] = ax.m[1];
-      S[(F::kF + 2 * b + 1) * NB] = ax.m[2];
-    }
-    S[F::kT * NB] = s.T;
-    S[F::kOm * NB] = mix.omega;
-    S[F::kCf * NB] = (SRC ? mix.omega + sum_rd * s.inv_sf : mix.omega) * s.sf;     // Eq. 42, Eq. 87
-    S[F::kTot * NB] = s.sf + sum_rd;                                               // Eq. 78
-    if (EN) {
-      R cU = mix.omega * s.sf * mix.U, c2 = mix.omega * s.sf, tot = mo.sg;
-      if (SRC) {
-        // source distribution with the post-reaction density and internal
-        // energy (Eq. 86): phi rho U gains dU, phi rho gains the sum of the sources
-        const R dU = (R)srcv[(size_t)(unsigned)M * N + n];
-        cU += dU;
-        c2 += sum_rd;
-        tot += dU + sum_rd * mix.hw2;
-      }
-      S[F::kRt * NB] = mix.RT;
-      S[F::kCu * NB] = cU;
-      S[F::kC2 * NB] = c2;
-      S[(F::kTot + 1) * NB] = tot;
-#pragma unroll
-      for (int b = 0; b < 3; ++b) S[(F::kDq + b) * NB] = mix.Dq[b];
+      for (int i = 0; i < 27; ++i) parked[i * NB] = f[i];
     }
   }
   __syncthreads();
@@ -363,99 +435,237 @@ __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
   auto put = [&](int i, const R& v) {
     if (live) dn[(size_t)(unsigned)i * N] = v;
   };
-  R w[3];
-#pragma unroll
-  for (int b = 0; b < 3; ++b) w[b] = S[(F::kW + b) * NB];
   if (l < M) {
-    // ---- species l (Eq. 21, Eq. 25) -----------------------------------------
-    const R* c = S + (F::kCo + F::kCoN * l) * NB;
-    const R sa = c[3 * NB], beta = c[4 * NB];
+    // ---- species l: its row of the diffusion system (Eq. 23, 24, 22, 26, 29) ------
+    bar_sync(1, NB * (M + 1));
+    R w[3], v[3], row[M], X[M];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) w[b] = S[(F::kW + b) * NB];
+    R h = R(0), hYl = R(0), beta, q, itk;
+#pragma unroll
+    for (int b = 0; b < M; ++b) {
+      const R hY = S[(F::kHY + b) * NB], t = hY * p.invDmm[l][b];      // zero on the diagonal
+      if (b == l) hYl = hY;
+      row[b] = -t;
+      h += t;
+    }
+    itk = p.knc[l] * S[F::kKT * NB];
+    q = R(1) / (R(1) + h);
+    beta = h * q;
+    const R hk = R(0.5) * itk, margin = R(1) + hk;
+    const bool tiny = Transport<R, 3, M>::unresolved(s0, S[F::kSS * NB], sabs);
+    const R isa = R(1) / s0;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) v[b] = (tiny ? R(0) : j0[b] * isa - w[b]) - hk * w[b];
+    if (ScalarTraits<R>::single) {
+      R rs = fabs(margin + h);
+#pragma unroll
+      for (int b = 0; b < M; ++b) rs += fabs(row[b]);
+      S[(F::kCond + l) * NB] = rs;
+      S[(F::kCond + M + l) * NB] = margin;
+    }
+#pragma unroll
+    for (int b = 0; b < M; ++b)
+      if (b == l) row[b] = margin + h;
+    bool fp64 = false;
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+      R* pv = S + (F::kPv + k * (M + 3)) * NB;
+      if (l == k) {
+        const R inv = R(1) / row[k];
+#pragma unroll
+        for (int c = k + 1; c < M; ++c) {
+          row[c] *= inv;
+          pv[c * NB] = row[c];
+        }
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          v[b] *= inv;
+          pv[(M + b) * NB] = v[b];
+        }
+      }
+      bar_sync(2, NB * M);
+      if (l != k) {
+        const R g = row[k];
+#pragma unroll
+        for (int c = k + 1; c < M; ++c) row[c] -= g * pv[c * NB];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) v[b] -= g * pv[(M + b) * NB];
+      }
+      if (ScalarTraits<R>::single && k == 0) {
+        // condition bound (R12): above it the system is solved in double
+        R amax = R(0), dmin = R(1e30);
+#pragma unroll
+        for (int b = 0; b < M; ++b) {
+          const R rs = S[(F::kCond + b) * NB], d = S[(F::kCond + M + b) * NB];
+          amax = rs > amax ? rs : amax;
+          dmin = d < dmin ? d : dmin;
+        }
+        fp64 = amax > p.kappa_thr * dmin;
+      }
+    }
+    if constexpr (ScalarTraits<R>::single) {
+      if (fp64) solve_row_fp64<R, M, EN, NB>(p, S, a.phi[n], l, v);
+      if (live && l == 0 && fp64) flag(a.status, 2);
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) S[(F::kV + 3 * l + b) * NB] = v[b];
+    bar_arrive(5, NB * (M + 1));
+    // ---- its difference moments and relaxation (Eq. 21, Eq. 25) --------------------
+    const R gd = q * itk, qY = R(2) * q * hYl;         // (1 - beta) Y_l C
     SpeciesTarget<R, 3> t;
     t.th = R(0.5) * p.Ra[l] * S[F::kT * NB];
-    t.gd = c[5 * NB];
-    t.gE = t.gd * sa;
-    t.qY = c[6 * NB];
-    t.cE = R(2) * beta * sa;
-    R total = sa;
+    t.gE = gd * s0;
+    t.cE = R(2) * beta * s0;
+    R total = s0;
     if (SRC) {
-      t.cE += c[7 * NB];                              // R^r = fdot^r dt
-      total += c[7 * NB];
+      const R rd = S[(F::kRd + l) * NB];
+      t.cE += rd;                                      // Eq. 89, R^r = fdot^r dt
+      total += rd;
     }
-    const R v[3] = {c[0], c[NB], c[2 * NB]};
     SpeciesAxes<R, 3> ax;
-    ax.set(w, v, sa, t.th);
-    R* D0 = S + F::kDelta * NB;
-    R own0[9], own1[9], own2[9];
-    ax.template delta<0>(own0);
-    ax.template delta<1>(own1);
-    ax.template delta<2>(own2);
+    ax.set(w, v, s0, t.th);
     {
-      R* d = D0 + 26 * l * NB;
-#pragma unroll
-      for (int e = 1; e < 9; ++e) d[(e - 1) * NB] = own0[e];
-#pragma unroll
-      for (int e = 0; e < 9; ++e) d[(8 + e) * NB] = own1[e];
-#pragma unroll
-      for (int e = 0; e < 9; ++e) d[(17 + e) * NB] = own2[e];
+      R* d = D0 + l * NB * F::kStride;
+      R m[9];
+      ax.template delta<0>(m);
+      store16<8>(d + F::kO0, m + 1);
+      ax.template delta<1>(m);
+      store16<9>(d + F::kO1, m);
+      ax.template delta<2>(m);
+      store16<9>(d + F::kO2, m);
     }
-    asm volatile("bar.sync 1, %0;\n" ::"n"(NB * M) : "memory");     // the species' groups
-    R D[M];
+    bar_sync(4, NB * M);
 #pragma unroll
-    for (int b = 0; b < M; ++b) D[b] = p.invDmm[l][b];              // zero on the diagonal
-    auto couple = [&](int e) {
-      R s = D[0] * D0[e * NB];
-#pragma unroll
-      for (int b = 1; b < M; ++b) s += D[b] * D0[(26 * b + e) * NB];
-      return s;
-    };
+    for (int b = 0; b < M; ++b) X[b] = (b == l) ? -gd : qY * p.invDmm[l][b];
     const R keep = R(1) - R(2) * beta;
-    R T2[9], T1[9], acc;
+    R T2[9], T1[9], m[9], acc;
+    couple<R, M, F::kStride, NB, 9>(D0 + F::kO2, X, T2);
+    couple<R, M, F::kStride, NB, 9>(D0 + F::kO1, X, T1);
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
-      T2[e] = t.template entry<2>(ax, w, e % 3, e / 3, own2[e], couple(17 + e));
-      T1[e] = t.template entry<1>(ax, w, e % 3, e / 3, own1[e], couple(8 + e));
+      T2[e] += t.template entry<2>(ax, w, e % 3, e / 3);
+      T1[e] += t.template entry<1>(ax, w, e % 3, e / 3);
     }
-    R m[9];
 #pragma unroll
     for (int e = 0; e < 9; ++e) m[e] = T2[e] - T1[e];
     acc = relax_dirs<R, 3, false>(get, -1, keep, m, nullptr, put);
 #pragma unroll
     for (int e = 0; e < 9; ++e) m[e] = T2[e] + T1[e];
     acc += relax_dirs<R, 3, false>(get, 1, keep, m, nullptr, put);
+    couple<R, M, F::kStride, NB, 8>(D0 + F::kO0, X, T1);
 #pragma unroll
     for (int e = 1; e < 9; ++e)
-      m[e] = t.template entry<0>(ax, w, e % 3, e / 3, own0[e], couple(e - 1)) - R(2) * T2[e];
+      m[e] = (T1[e - 1] + t.template entry<0>(ax, w, e % 3, e / 3)) - R(2) * T2[e];
     acc += relax_dirs<R, 3, false>(get, 0, keep, m, nullptr, put);
     put(13, total - acc);
-  } else {
-    R m[3][9], ex[3] = {R(0), R(0), R(0)}, total;
-    if (l == M) {
-      // ---- momentum (Eq. 42, Eq. 44, Eq. 87) -----------------------------------
-      Axis<R> ax[3];
-#pragma unroll
-      for (int b = 0; b < 3; ++b) ax[b].set(R(1), S[(F::kF + 2 * b) * NB], S[(F::kF + 2 * b + 1) * NB]);
-      product_moments<R, 3>(S[F::kCf * NB], ax, m);
-      total = S[F::kTot * NB];
-    } else {
-      // ---- energy (Eq. 43, Eq. 51, Eq. 54, Eq. 88) ------------------------------
-      energy_moments<R, 3>(S[F::kCu * NB], S[F::kC2 * NB], S[F::kRt * NB], w, m);
-#pragma unroll
-      for (int b = 0; b < 3; ++b) ex[b] = S[(F::kDq + b) * NB];
-      total = S[(F::kTot + 1) * NB];
-    }
-    const R keep = R(1) - S[F::kOm * NB];
-    R t[9], acc;
-#pragma unroll
-    for (int e = 0; e < 9; ++e) t[e] = m[2][e] - m[1][e];
-    acc = relax_dirs<R, 3, true>(get, -1, keep, t, ex, put);
-#pragma unroll
-    for (int e = 0; e < 9; ++e) t[e] = m[2][e] + m[1][e];
-    acc += relax_dirs<R, 3, true>(get, 1, keep, t, ex, put);
-#pragma unroll
-    for (int e = 1; e < 9; ++e) t[e] = m[0][e] - R(2) * m[2][e];
-    acc += relax_dirs<R, 3, true>(get, 0, keep, t, ex, put);
-    put(13, total - acc);
+    return;
   }
+  R m[3][9], ex[3] = {R(0), R(0), R(0)}, total, keep;
+  if (l == L - 1) {
+    // ---- last group: state, then mixture (and the energy lattice) -------------------
+    Moments<R, 3, M, EN, true> mo;
+#pragma unroll
+    for (int k = 0; k < M; ++k) mo.sa[k] = S[F::kSp * k * NB];
+    mo.sf = S[F::kMo * NB];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) mo.jf[b] = S[(F::kMo + 1 + b) * NB];
+    if (EN) mo.sg = s0;
+    State<R, 3, M> s;
+    s.template from_moments<EN, true>(p, mo, phi, Tf);
+    const R inv_phi = R(1) / s.phi;
+    const R kT = s.T * rsqrt_<R>(s.T) * inv_phi, hC = R(0.5) * p.Kc * s.sf * kT;      // as in Transport
+#pragma unroll
+    for (int b = 0; b < 3; ++b) S[(F::kW + b) * NB] = s.w[b];
+    S[F::kT * NB] = s.T;
+    S[F::kSS * NB] = s.ss;
+    S[F::kKT * NB] = p.knudsen ? kT : R(0);
+#pragma unroll
+    for (int k = 0; k < M; ++k) S[(F::kHY + k) * NB] = hC * s.Y[k];
+    bar_arrive(1, NB * (M + 1));
+    if (live && bad_state(s, inv_phi)) flag(a.status, 1);
+    Grad<R, 3, M, EN> gr;
+    gr.divu = S[F::kU * NB] + S[(F::kU + 1) * NB] + S[(F::kU + 2) * NB];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) gr.dPi[b] = S[(F::kU + 3 + b) * NB];
+    R itk[M], sum_rd = R(0);
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+      itk[k] = p.knudsen ? p.knc[k] * kT : R(0);
+      if (SRC) sum_rd += S[(F::kRd + k) * NB];
+    }
+    Mixture<R, 3> mix;
+    mix.template scalars<M, EN>(p, s, inv_phi, gr.divu);
+    bar_sync(5, NB * (M + 1));
+    R v[M][3], vbar[3];
+#pragma unroll
+    for (int k = 0; k < M; ++k)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) v[k][b] = S[(F::kV + 3 * k + b) * NB];
+    mix.template force<M>(s, itk, v, vbar);
+    const R cf = (SRC ? mix.omega + sum_rd * s.inv_sf : mix.omega) * s.sf;            // Eq. 42, Eq. 87
+    Axis<R> F3[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) mix.momentum_axis(s.w[b], s.inv_sf, b, gr.dPi[b], F3[b]);
+    keep = R(1) - mix.omega;
+    if constexpr (EN) {
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        S[(F::kF + 2 * b) * NB] = F3[b].m[1];
+        S[(F::kF + 2 * b + 1) * NB] = F3[b].m[2];
+      }
+      S[F::kOm * NB] = mix.omega;
+      S[F::kCf * NB] = cf;
+      S[F::kTot * NB] = s.sf + sum_rd;                                                // Eq. 78
+      bar_arrive(3, 2 * NB);
+      // ---- energy (Eq. 43, Eq. 51, Eq. 54, Eq. 88) --------------------------------
+      int e = F::kMo + 4;
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        mo.q[b] = j0[b];
+#pragma unroll
+        for (int c = b; c < 3; ++c) mo.Pt[b][c] = mo.Pt[c][b] = S[(e++) * NB];
+#pragma unroll
+        for (int k = 0; k < M; ++k) gr.dY[k][b] = S[(F::kDY + 3 * k + b) * NB];
+      }
+      mix.template heat<M, EN>(p, mo, s, v, vbar, gr);
+      R cU = mix.omega * s.sf * mix.U, c2 = mix.omega * s.sf;
+      total = mo.sg;
+      if (SRC) {
+        // source distribution with the post-reaction density and internal
+        // energy (Eq. 86): phi rho U gains dU, phi rho gains the sum of the sources
+        cU += dU;
+        c2 += sum_rd;
+        total += dU + sum_rd * mix.hw2;
+      }
+#pragma unroll
+      for (int b = 0; b < 3; ++b) ex[b] = mix.Dq[b];
+      energy_moments<R, 3>(cU, c2, mix.RT, s.w, m);
+    } else {
+      total = s.sf + sum_rd;
+      product_moments<R, 3>(cf, F3, m);
+    }
+  } else {
+    // ---- momentum (Eq. 42, Eq. 44, Eq. 87) -----------------------------------------
+    bar_sync(3, 2 * NB);
+    Axis<R> F3[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) F3[b].set(R(1), S[(F::kF + 2 * b) * NB], S[(F::kF + 2 * b + 1) * NB]);
+    product_moments<R, 3>(S[F::kCf * NB], F3, m);
+    total = S[F::kTot * NB];
+    keep = R(1) - S[F::kOm * NB];
+  }
+  R t[9], acc;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) t[e] = m[2][e] - m[1][e];
+  acc = relax_dirs<R, 3, true>(get, -1, keep, t, ex, put);
+#pragma unroll
+  for (int e = 0; e < 9; ++e) t[e] = m[2][e] + m[1][e];
+  acc += relax_dirs<R, 3, true>(get, 1, keep, t, ex, put);
+#pragma unroll
+  for (int e = 1; e < 9; ++e) t[e] = m[0][e] - R(2) * m[2][e];
+  acc += relax_dirs<R, 3, true>(get, 0, keep, t, ex, put);
+  put(13, total - acc);
 }
 
 }  // namespace lbm
