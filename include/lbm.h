@@ -322,8 +322,9 @@ int lbm_get_timing(lbm_ctx* ctx, double* ms_by_kind /* [3] */, long long* launch
  * asynchronous copies, 5 a fused halo tile, 6-7 the staged two-pass form,
  * 8-9 the row march staged by bulk tensor copies (TMA; on lattices whose
  * rows are not a multiple of 16 bytes they run the per-thread-copy march of
- * the same tile shape, variants 2 and 0), 10-12 the single-launch form on
- * tiles of 8 x 4, 16 x 8 and 32 x 4 nodes with the populations in registers.
+ * the same tile shape, variants 2 and 0), 10 the single-launch form on tiles
+ * of 8 x 4 nodes with one warp per lattice, 11-12 the single-launch form on
+ * tiles of 16 x 8 and 32 x 4 nodes with a node's populations in one thread.
  * D3Q27: every form is the two-pass step split by lattice (one warp per
  * lattice of 32 nodes); the indices select the registers a thread may use
  * (0: one resident block per SM, 1: two, 2: three, 3: four; 4 and 5 the
@@ -331,7 +332,7 @@ int lbm_get_timing(lbm_ctx* ctx, double* ms_by_kind /* [3] */, long long* launch
  * computes the same step (the gradient stencil is summed in different
  * orders, so the forms agree to rounding).  New contexts use variant 5 in
  * 3-D and, in 2-D, variant 8 on FP32 lattices of at least 2^18 nodes with nx a
- * multiple of 4 and no reservoir face, else tiles (10 below 8192 nodes, above
+ * multiple of 4 and no reservoir face, else tiles (10 up to 9728 nodes, above
  * that 12 in FP32 and 11 in FP64; lattices of one or two rows with 8192 nodes
  * or more: the two-pass form); batches use variant 10.  The adjoint's
  * forward and recompute steps use the context's form.  lbm_autotune times

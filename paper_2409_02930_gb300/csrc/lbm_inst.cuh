@@ -3,7 +3,7 @@
 #include "lbm_fused.cuh"
 #include "lbm_march2d.cuh"
 #include "lbm_ops.h"
-#include "lbm_split3d.cuh"
+#include "lbm_split2d.cuh"
 #include "lbm_staged.cuh"
 
 namespace lbm {
@@ -79,6 +79,13 @@ struct Launch {
     if ((p.ny + TY - 1) / TY > 65535) return -1;
     if constexpr (D == 2)
       k_tile2d<R, M, EN, TX, TY, MINB><<<dim3((p.nx + TX - 1) / TX, (p.ny + TY - 1) / TY), TX * TY, 0, s>>>(p, it, a);
+    return 0;
+  }
+  // tiles split by lattice, one warp each
+  static int split2d(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
+    if ((p.ny + 3) / 4 > 65535) return -1;
+    if constexpr (D == 2)
+      k_split2d<R, M, EN><<<dim3((p.nx + 7) / 8, (p.ny + 3) / 4), 32 * (L + 1), 0, s>>>(p, it, a);
     return 0;
   }
   // pipelined 2-D step (cp.async staging), TX columns marching SEG rows
@@ -157,7 +164,7 @@ struct Launch {
         case 7: return staged<128>(p, it, a, s);
         case 8: return march2d_tma<32, 8, 1, 1>(p, it, a, s);
         case 9: return march2d_tma<64, 8, 1, 1>(p, it, a, s);
-        case 10: return tile2d<8, 4, 1>(p, it, a, s);
+        case 10: return split2d(p, it, a, s);
         case 11: return tile2d<16, 8, sizeof(R) == 4 ? 3 : 1>(p, it, a, s);
         case 12: return tile2d<32, 4, sizeof(R) == 4 ? 3 : 1>(p, it, a, s);
         default: return -1;

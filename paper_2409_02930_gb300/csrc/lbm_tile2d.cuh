@@ -17,10 +17,10 @@
 // a bare copy of the state 14.0 us, pulls and halo without arithmetic 20.7 us,
 // the step 30.4 us at 12 warps per SM; 128 registers and 16 warps, 256-node
 // blocks, and two nodes per thread in packed FP32 arithmetic were no faster);
-// in FP64 the FP64 pipe; on small lattices one block's latency.  Against the
-// form that served each size before: 256 x 4 FP64 109 -> 33 us per step,
-// 64 x 40 FP32 29 -> 4.9, 512 x 384 with reservoirs 158 -> 24.9, 701 x 523 with
-// walls 73 -> 44, 512 x 512 FP64 1010 -> 536.
+// in FP64 the FP64 pipe.  Against the form that served each size before:
+// 512 x 384 FP32 with reservoirs 158 -> 24.9 us per step, 701 x 523 with walls
+// 73 -> 44, 512 x 512 FP64 1010 -> 536.  Lattices of a few thousand nodes are
+// bound by one block's latency and run split by lattice (lbm_split2d.cuh).
 #pragma once
 
 #include "lbm_twopass.cuh"

@@ -162,3 +162,23 @@ def test_adjoint_on_degenerate_lattices(L, nx, ny, bc):
         e[n] = eps
         fd[n] = (J(wl.porosity + e) - J(wl.porosity - e)) / (2 * eps)
     assert np.max(np.abs(grad - fd)) <= 1e-6 * np.max(np.abs(fd)) + 1e-12
+
+
+@pytest.mark.parametrize("nx,ny", [(8, 4), (37, 11)])
+def test_split_2d_solves_in_double_above_the_bound(L, nx, ny):
+    """The lattice-split tile (form 10) with every node's diffusion system sent
+    to the FP64 solve, against the oracle within the FP32 bound."""
+    wl = slab(nx, ny, W.BC_PERIODIC)
+    o = oracle.Oracle(wl)
+    o.step(STEPS)
+    g = L.Lattice(wl, precision=L.LBM_FP32, kappa_threshold=1e-30)
+    g.set_variant(10)
+    g.step(STEPS)
+    g.sync()
+    assert worst(g.populations(), o.pops()) < FP32_BOUND
+    g.close()
+
+
+def test_split_2d_six_species(L):
+    """Six species on a two-dimensional lattice, form 10 and the tiles."""
+    check_forms(L, anode(19, 6, 1), range(10, 13))
