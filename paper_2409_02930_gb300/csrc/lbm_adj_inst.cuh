@@ -28,22 +28,22 @@ struct AdjLaunch {
   static int grid(int n, int b) { return (n + b - 1) / b; }
   static int done() { return cudaGetLastError() == cudaSuccess ? 0 : -1; }
   static int fields(const Params<B>& p, const InletTables<B>& it, const AdjArgs<B>& a, cudaStream_t s) {
-    k_adj_fields<B, M, EN><<<grid(p.N, 128), 128, 0, s>>>(p, it, a);
+    launch_after(k_adj_fields<B, M, EN>, grid(p.N, 128), 128, 0, s, p, it, a);
     return done();
   }
   static int collide(const Params<B>& p, const InletTables<B>& it, const AdjArgs<B>& a, cudaStream_t s) {
-    k_adj_collide<B, M, EN><<<grid(p.N, 64), 64, 0, s>>>(p, it, a);
+    launch_after(k_adj_collide<B, M, EN>, grid(p.N, 64), 64, 0, s, p, it, a);
     return done();
   }
   static int macro(const Params<B>& p, const AdjArgs<B>& a, bool seed, cudaStream_t s) {
-    if (seed) k_adj_macro<B, M, EN, false><<<grid(p.N, 128), 128, 0, s>>>(p, a);
-    else k_adj_macro<B, M, EN, true><<<grid(p.N, 128), 128, 0, s>>>(p, a);
+    if (seed) launch_after(k_adj_macro<B, M, EN, false>, grid(p.N, 128), 128, 0, s, p, a);
+    else launch_after(k_adj_macro<B, M, EN, true>, grid(p.N, 128), 128, 0, s, p, a);
     return done();
   }
   static int ghost(const Params<B>& p, const InletTables<B>& it, const AdjArgs<B>& a, cudaStream_t s) {
     Params<Dual<B, 3>> pd;
     params_cast(p, pd);
-    k_adj_ghost<B, M, EN><<<dim3(grid(p.ny, 32), p.nx > 3 ? 2 : 1), 32, 0, s>>>(p, it, a, pd);
+    launch_after(k_adj_ghost<B, M, EN>, dim3(grid(p.ny, 32), p.nx > 3 ? 2 : 1), 32, 0, s, p, it, a, pd);
     return done();
   }
   static void seed_flux(const Params<B>& p, const AdjArgs<B>& a, int species, int axis, int xo, double w,

@@ -60,6 +60,7 @@ struct AdjArgs {
 // Macro fields of f^n and the sums behind them.
 template <class B, int M, bool EN>
 __global__ void __launch_bounds__(128) k_adj_fields(Params<B> p, InletTables<B> it, AdjArgs<B> a) {
+  after_previous();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= p.N) return;
   const size_t N = p.N;
@@ -85,6 +86,7 @@ __global__ void __launch_bounds__(128) k_adj_fields(Params<B> p, InletTables<B> 
 template <class B, int M, bool EN>
 __global__ void __launch_bounds__(64) k_adj_collide(Params<B> p, InletTables<B> it, AdjArgs<B> a) {
   constexpr int L = n_lat<2, M, EN>(), REST = 4;
+  after_previous();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= p.N) return;
   const int N = p.N;
@@ -152,6 +154,7 @@ __global__ void __launch_bounds__(64) k_adj_collide(Params<B> p, InletTables<B> 
 // population stays in Pbar for k_adj_ghost.
 template <class B, int M, bool EN, bool MACRO>
 __global__ void __launch_bounds__(128) k_adj_macro(Params<B> p, AdjArgs<B> a) {
+  after_previous();
   constexpr int L = n_lat<2, M, EN>();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= p.N) return;
@@ -262,6 +265,7 @@ template <class B, int M, bool EN>
 __global__ void __launch_bounds__(32) k_adj_ghost(Params<B> p, InletTables<B> it, AdjArgs<B> a,
                                                   const __grid_constant__ Params<Dual<B, 3>> pd) {
   using T = Dual<B, 3>;
+  after_previous();
   const int y = blockIdx.x * blockDim.x + threadIdx.x;
   if (y >= p.ny) return;
   const size_t N = p.N;

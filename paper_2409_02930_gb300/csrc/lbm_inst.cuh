@@ -34,7 +34,7 @@ struct Launch {
   static int macro3(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, R* aux, cudaStream_t s) {
     if constexpr (D == 3) {
       constexpr size_t smem = split_smem_bytes<R, M, EN>(NB, false, false);
-      k_macro3<R, M, EN, NB, AUX><<<(p.N + NB - 1) / NB, NB * L, smem, s>>>(p, it, a, aux);
+      launch_after(k_macro3<R, M, EN, NB, AUX>, (p.N + NB - 1) / NB, NB * L, smem, s, p, it, a, aux);
     }
     return 0;
   }
@@ -46,7 +46,7 @@ struct Launch {
       auto kern = k_collide3<R, M, EN, NB, SRC, MINB, PARK>;
       static bool done = false;
       if (configure(kern, smem, done)) return -1;
-      kern<<<(p.N + NB - 1) / NB, NB * L, smem, s>>>(p, it, a, src);
+      launch_after(kern, (p.N + NB - 1) / NB, NB * L, smem, s, p, it, a, src);
     }
     return 0;
   }
@@ -54,11 +54,11 @@ struct Launch {
   static constexpr bool kPark = sizeof(R) == 4;
   static void macro(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
     if constexpr (D == 3) macro3<false>(p, it, a, nullptr, s);
-    else k_macro<R, D, M, EN><<<grid(p.N), block(p.N), 0, s>>>(p, it, a);
+    else launch_after(k_macro<R, D, M, EN>, grid(p.N), block(p.N), 0, s, p, it, a);
   }
   static void collide(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
     if constexpr (D == 3) collide3<false, kMinB, kPark>(p, it, a, nullptr, s);
-    else k_collide<R, D, M, EN><<<grid(p.N), block(p.N), 0, s>>>(p, it, a);
+    else launch_after(k_collide<R, D, M, EN>, grid(p.N), block(p.N), 0, s, p, it, a);
   }
   // fused step, shared-memory halo ring, tile TX x TY marching SEG planes
   template <int TX, int TY, int SEG>
@@ -78,14 +78,15 @@ struct Launch {
   static int tile2d(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
     if ((p.ny + TY - 1) / TY > 65535) return -1;
     if constexpr (D == 2)
-      k_tile2d<R, M, EN, TX, TY, MINB><<<dim3((p.nx + TX - 1) / TX, (p.ny + TY - 1) / TY), TX * TY, 0, s>>>(p, it, a);
+      launch_after(k_tile2d<R, M, EN, TX, TY, MINB>, dim3((p.nx + TX - 1) / TX, (p.ny + TY - 1) / TY), TX * TY, 0, s, p,
+                   it, a);
     return 0;
   }
   // tiles split by lattice, one warp each
   static int split2d(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
     if ((p.ny + 3) / 4 > 65535) return -1;
     if constexpr (D == 2)
-      k_split2d<R, M, EN><<<dim3((p.nx + 7) / 8, (p.ny + 3) / 4), 32 * (L + 1), 0, s>>>(p, it, a);
+      launch_after(k_split2d<R, M, EN>, dim3((p.nx + 7) / 8, (p.ny + 3) / 4), 32 * (L + 1), 0, s, p, it, a);
     return 0;
   }
   // pipelined 2-D step (cp.async staging), TX columns marching SEG rows
@@ -104,7 +105,7 @@ struct Launch {
         static bool done[2] = {false, false};
         if (configure(kern, smem, done[inlet ? 1 : 0])) return -1;
         dim3 g((p.nx + TX - 3) / (TX - 2), (p.ny + SEG - 1) / SEG, 1);
-        kern<<<g, TX, smem, s>>>(p, it, a, TmaMaps{});
+        launch_after(kern, g, TX, smem, s, p, it, a, TmaMaps{});
         return 0;
       }
     }
@@ -130,7 +131,7 @@ struct Launch {
         static bool done[2] = {false, false};
         if (configure(kern, smem, done[inlet ? 1 : 0])) return -1;
         dim3 g((p.nx + TX - 3) / (TX - 2), (p.ny + SEG - 1) / SEG, 1);
-        kern<<<g, TX, smem, s>>>(p, it, a, tm);
+        launch_after(kern, g, TX, smem, s, p, it, a, tm);
         return 0;
       }
     }
@@ -198,7 +199,7 @@ struct Launch {
       R* aux = a.mac + (size_t)(2 * D + M) * p.N;
       macro3<true>(p, it, a, aux, s);
       if (p.N <= source_warp_nodes) {
-        k_source_warp<R, M><<<p.N, 32, 0, s>>>(p.N, aux, a.phi, a.status, ra);
+        launch_after(k_source_warp<R, M>, p.N, 32, 0, s, p.N, aux, a.phi, a.status, ra);
       } else if (p.N <= source_wide_nodes) {
         k_source<R, M, 1><<<(p.N + 127) / 128, 128, 0, s>>>(p.N, aux, a.phi, a.status, ra);
       } else {

@@ -2,6 +2,7 @@
 // populations.
 #pragma once
 
+#include "lbm_launch.h"
 #include "lbm_node.cuh"
 
 namespace lbm {

@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(TX, MINB)
     __syncthreads();
   }
 
+  after_previous();
   auto issue = [&](int row) {
     const int y = modp(row, p.ny);
     if (TMA && bulk) {

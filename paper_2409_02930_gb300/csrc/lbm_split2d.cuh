@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(32 * (M + 2 + (EN ? 1 : 0))) k_split2d(Params<
   // last), 7 mixture ready (last to momentum)
   __shared__ R mac[T::NF * PN];
   __shared__ R sh[F::kAll * 32];
+  after_previous();
   const int lane = threadIdx.x & 31, l = group_of<32>();
   R* S = sh + lane;
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;

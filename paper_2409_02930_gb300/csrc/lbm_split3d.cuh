@@ -247,9 +247,10 @@ __device__ __forceinline__ void pull_lattice(const Params<R>& p, const InletTabl
 // sums and the temperature that the surface source reads.
 template <class R, int M, bool EN, int NB, bool AUX>
 __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0))) k_macro3(Params<R> p, InletTables<R> it, StepArgs<R> a,
-                                                                       R* __restrict__ aux) {
+                                                                       R* aux) {
   using F = SplitFields<R, M, EN>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   const int lane = threadIdx.x % NB, l = group_of<NB>();
   R* S = reinterpret_cast<R*>(smem_raw) + lane;
   const int n = min((int)(blockIdx.x * NB) + lane, p.N - 1);
@@ -358,13 +359,14 @@ __device__ __noinline__ void solve_row_fp64(const Params<R>& p, const R* S, R ph
 // the fluid internal energy).
 template <class R, int M, bool EN, int NB, bool SRC, int MINB, bool PARK>
 __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
-    k_collide3(Params<R> p, InletTables<R> it, StepArgs<R> a, const double* __restrict__ srcv) {
+    k_collide3(Params<R> p, InletTables<R> it, StepArgs<R> a, const double* srcv) {
   using F = SplitFields<R, M, EN>;
   constexpr int L = M + 1 + (EN ? 1 : 0);
   // barriers: 0 all; 1 state ready (last group to the species), 2 pivot rows
   // (species), 3 mixture ready (last group to the momentum group), 4
   // difference moments (species), 5 v ready (species to the last group)
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   const int lane = threadIdx.x % NB, l = group_of<NB>();
   R* S = reinterpret_cast<R*>(smem_raw) + lane;
   R* D0 = reinterpret_cast<R*>(smem_raw) + F::kAll * NB + lane * F::kStride;

@@ -308,7 +308,7 @@ struct ReactArgs {
 // Surface source of every node, from the species sums and temperatures that
 // the macro-field pass left in aux ([M + 1][N]).
 template <class R, int M, int MINB>
-__global__ void __launch_bounds__(128, MINB) k_source(int N, const R* __restrict__ aux, const R* __restrict__ phi,
+__global__ void __launch_bounds__(128, MINB) k_source(int N, const R* aux, const R* __restrict__ phi,
                                                 int* status, ReactArgs ra) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
@@ -347,7 +347,7 @@ constexpr int source_wide_nodes = 152 * 128 * 2;
 // over a species' steps in the same order, and the concentrations follow the
 // extents by increments.  12 x 2 x 2 anode in FP64: see the figures above.
 template <class RK, int M>
-__global__ void __launch_bounds__(32) k_source_warp(int N, const RK* __restrict__ aux, const RK* __restrict__ phi,
+__global__ void __launch_bounds__(32) k_source_warp(int N, const RK* aux, const RK* __restrict__ phi,
                                                     int* status, ReactArgs ra) {
   constexpr int NSX = MMAX + SMAX;
   constexpr unsigned FULL = 0xffffffffu;
@@ -375,6 +375,7 @@ __global__ void __launch_bounds__(32) k_source_warp(int N, const RK* __restrict_
         ro[j] = mc.rord[lane][j];
       }
   }
+  after_previous();                                         // the mechanism is constant, the fields are not
   const int n = blockIdx.x;
   const double ph = (double)phi[n], T = (double)aux[(size_t)M * N + n];
   const double dphi = mc.dphi_field ? mc.dphi_field[n] : mc.dphi;

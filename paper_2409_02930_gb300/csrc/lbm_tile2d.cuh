@@ -131,6 +131,7 @@ template <class R, int M, bool EN, int TX, int TY, int MINB>
 __global__ void __launch_bounds__(TX * TY, MINB) k_tile2d(Params<R> p, InletTables<R> it, StepArgs<R> a) {
   using T = TileShape<R, M, EN, TX, TY>;
   __shared__ R mac[T::NF * T::PN];
+  after_previous();
   tile2d_step<R, M, EN, TX, TY>(p, it, a, blockIdx.x * TX, blockIdx.y * TY, mac);
 }
 

@@ -41,6 +41,7 @@ LBM_HD void macro_node(const Params<R>& p, const InletTables<R>& it, const StepA
 
 template <class R, int D, int M, bool EN>
 __global__ void __launch_bounds__(256) k_macro(Params<R> p, InletTables<R> it, StepArgs<R> a) {
+  after_previous();
   int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n < p.N) macro_node<R, D, M, EN>(p, it, a, n);
 }
@@ -67,6 +68,7 @@ LBM_HD void collide_node(const Params<R>& p, const InletTables<R>& it, const Ste
 
 template <class R, int D, int M, bool EN>
 __global__ void __launch_bounds__(256) k_collide(Params<R> p, InletTables<R> it, StepArgs<R> a) {
+  after_previous();
   int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n < p.N) collide_node<R, D, M, EN>(p, it, a, n);
 }
