@@ -28,17 +28,19 @@ struct Launch {
   // small lattices take small blocks, so that they spread over the SMs
   static int block(int N) { return N < 152 * 512 ? 64 : 256; }
   static int grid(int N) { return (N + block(N) - 1) / block(N); }
-  // 3-D: the step split by lattice, NB = 32 nodes and one warp per lattice in a block
-  static constexpr int NB = 32, L = M + 1 + (EN ? 1 : 0);
-  template <bool AUX>
+  // 3-D: the step split by lattice, NB = 32 nodes and one warp per lattice in a
+  // block; small FP64 lattices take 8 or 16 nodes and several species per warp
+  static constexpr int L = M + 1 + (EN ? 1 : 0);
+  template <bool AUX, int NB>
   static int macro3(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, R* aux, cudaStream_t s) {
     if constexpr (D == 3) {
       constexpr size_t smem = split_smem_bytes<R, M, EN>(NB, false, false);
-      launch_after(k_macro3<R, M, EN, NB, AUX>, (p.N + NB - 1) / NB, NB * L, smem, s, p, it, a, aux);
+      launch_after(k_macro3<R, M, EN, NB, AUX>, (p.N + NB - 1) / NB, SplitThreads<NB, M, EN>::kAll, smem, s, p, it, a,
+                   aux);
     }
     return 0;
   }
-  template <bool SRC, int MINB, bool PARK>
+  template <bool SRC, int NB, int MINB, bool PARK>
   static int collide3(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, const double* src,
                       cudaStream_t s) {
     if constexpr (D == 3) {
@@ -46,18 +48,35 @@ struct Launch {
       auto kern = k_collide3<R, M, EN, NB, SRC, MINB, PARK>;
       static bool done = false;
       if (configure(kern, smem, done)) return -1;
-      launch_after(kern, (p.N + NB - 1) / NB, NB * L, smem, s, p, it, a, src);
+      launch_after(kern, (p.N + NB - 1) / NB, SplitThreads<NB, M, EN>::kAll, smem, s, p, it, a, src);
     }
     return 0;
   }
   static constexpr int kMinB = 2;
   static constexpr bool kPark = sizeof(R) == 4;
+  template <bool AUX>
+  static int macro_any(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, R* aux, cudaStream_t s) {
+    if constexpr (sizeof(R) == 8) {
+      if (p.N <= split3d_nodes8) return macro3<AUX, 8>(p, it, a, aux, s);
+      if (p.N <= split3d_nodes16) return macro3<AUX, 16>(p, it, a, aux, s);
+    }
+    return macro3<AUX, 32>(p, it, a, aux, s);
+  }
+  template <bool SRC>
+  static int collide_any(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, const double* src,
+                         cudaStream_t s) {
+    if constexpr (sizeof(R) == 8) {
+      if (p.N <= split3d_nodes8) return collide3<SRC, 8, 1, false>(p, it, a, src, s);
+      if (p.N <= split3d_nodes16) return collide3<SRC, 16, 1, false>(p, it, a, src, s);
+    }
+    return collide3<SRC, 32, kMinB, kPark>(p, it, a, src, s);
+  }
   static void macro(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
-    if constexpr (D == 3) macro3<false>(p, it, a, nullptr, s);
+    if constexpr (D == 3) macro_any<false>(p, it, a, nullptr, s);
     else launch_after(k_macro<R, D, M, EN>, grid(p.N), block(p.N), 0, s, p, it, a);
   }
   static void collide(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
-    if constexpr (D == 3) collide3<false, kMinB, kPark>(p, it, a, nullptr, s);
+    if constexpr (D == 3) collide_any<false>(p, it, a, nullptr, s);
     else launch_after(k_collide<R, D, M, EN>, grid(p.N), block(p.N), 0, s, p, it, a);
   }
   // fused step, shared-memory halo ring, tile TX x TY marching SEG planes
@@ -171,14 +190,15 @@ struct Launch {
         default: return -1;
       }
     } else {
-      macro3<false>(p, it, a, nullptr, s);
+      if (v < 3) macro3<false, 32>(p, it, a, nullptr, s);
+      else macro_any<false>(p, it, a, nullptr, s);
       switch (v) {
-        case 0: return collide3<false, 1, false>(p, it, a, nullptr, s);
-        case 1: return collide3<false, 2, false>(p, it, a, nullptr, s);
-        case 2: return collide3<false, sizeof(R) == 4 ? 3 : 2, false>(p, it, a, nullptr, s);
+        case 0: return collide3<false, 32, 1, false>(p, it, a, nullptr, s);
+        case 1: return collide3<false, 32, 2, false>(p, it, a, nullptr, s);
+        case 2: return collide3<false, 32, sizeof(R) == 4 ? 3 : 2, false>(p, it, a, nullptr, s);
         case 3:
         case 4:
-        case 5: return collide3<false, kMinB, kPark>(p, it, a, nullptr, s);
+        case 5: return collide_any<false>(p, it, a, nullptr, s);
         default: return -1;
       }
     }
@@ -197,7 +217,7 @@ struct Launch {
                           cudaStream_t s) {
     if constexpr (has_react) {
       R* aux = a.mac + (size_t)(2 * D + M) * p.N;
-      macro3<true>(p, it, a, aux, s);
+      macro_any<true>(p, it, a, aux, s);
       if (p.N <= source_warp_nodes) {
         launch_after(k_source_warp<R, M>, p.N, 32, 0, s, p.N, aux, a.phi, a.status, ra);
       } else if (p.N <= source_wide_nodes) {
@@ -209,7 +229,7 @@ struct Launch {
   }
   static void react_collide(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, const ReactArgs& ra,
                             cudaStream_t s) {
-    if constexpr (has_react) collide3<true, kMinB, kPark>(p, it, a, ra.src, s);
+    if constexpr (has_react) collide_any<true>(p, it, a, ra.src, s);
   }
   static Ops<R> ops() {
     return Ops<R>{macro, collide, fused, n_variants, init, moments, has_react ? react_macro : nullptr,

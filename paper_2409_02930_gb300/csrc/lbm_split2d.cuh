@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(32 * (M + 2 + (EN ? 1 : 0))) k_split2d(Params<
   __shared__ R mac[T::NF * PN];
   __shared__ R sh[F::kAll * 32];
   after_previous();
-  const int lane = threadIdx.x & 31, l = group_of<32>();
+  const int lane = threadIdx.x & 31, l = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0);
   R* S = sh + lane;
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
   const int tx = lane % TX, ty = lane / TX;

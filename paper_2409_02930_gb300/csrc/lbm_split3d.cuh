@@ -61,12 +61,35 @@ constexpr size_t split_smem_bytes(int NB, bool collide, bool park) {
          (collide ? F::kAll + M * F::kStride + (park ? 27 * (M + 1 + (EN ? 1 : 0)) : 0) : F::kSums);
 }
 
-// lattice of this thread's warp, known to the compiler as one value per warp
-// (addresses of the lattice's planes then come from uniform registers)
-template <int NB>
+// FP64 lattices up to these many nodes take blocks of 8 and of 16 nodes.  An
+// FP64 instruction of a warp holds its SM's only FP64 pipe for 16 cycles, so a
+// small lattice is bound by the pipes of the few SMs that its blocks reach:
+// 48 nodes in blocks of 32 ran 16 warps on two SMs, in blocks of 8 four warps on
+// each of six.  Larger lattices lose, since more warps carry the same nodes.
+// us per step with 32 / 16 / 8 nodes in a block: 12 x 2 x 2 88 / 63 / 56, 512
+// nodes 85 / 61 / 54, 1,024 85 / 61 / 74, 4,096 152 / 123 / 137, 8,192 153 / 201 /
+// 238; reactive 12 x 2 x 2 141 / 115 / 107.  FP32 gains nothing (12 x 2 x 2 9.5 /
+// 10.1 / 9.4, 4,096 nodes 12.9 / 13.4 / 16.8).
+constexpr int split3d_nodes8 = 152 * 4, split3d_nodes16 = 152 * 32;
+
+// Threads of a block of NB nodes: the species' groups of NB threads first,
+// rounded up to whole warps, then the momentum and the energy group in warps of
+// their own.  With NB < 32 a warp holds several species, and threads beyond the
+// last species or node repeat another thread's work (same values to the same
+// places).
+template <int NB, int M, bool EN>
+struct SplitThreads {
+  static constexpr int kSp = (M * NB + 31) / 32 * 32, kOne = NB < 32 ? 32 : NB, kAll = kSp + kOne * (EN ? 2 : 1);
+};
+
+// lattice of this thread; where a warp holds one lattice, known to the compiler
+// as one value per warp (addresses of its planes then come from uniform registers)
+template <int NB, int M, bool EN>
 __device__ __forceinline__ int group_of() {
-  static_assert(NB % 32 == 0, "a warp holds one lattice");
-  return __shfl_sync(0xffffffffu, (int)threadIdx.x / NB, 0);
+  using B = SplitThreads<NB, M, EN>;
+  const int t = (int)threadIdx.x;
+  if (NB % 32 == 0) return __shfl_sync(0xffffffffu, t / NB, 0);
+  return t < B::kSp ? min(t / NB, M - 1) : M + (t - B::kSp) / B::kOne;
 }
 
 // named barriers among `n` threads of the block
@@ -246,12 +269,12 @@ __device__ __forceinline__ void pull_lattice(const Params<R>& p, const InletTabl
 // First pass: macro fields of NB nodes (u, Pi, Y_a), and with AUX the species
 // sums and the temperature that the surface source reads.
 template <class R, int M, bool EN, int NB, bool AUX>
-__global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0))) k_macro3(Params<R> p, InletTables<R> it, StepArgs<R> a,
-                                                                       R* aux) {
+__global__ void __launch_bounds__(SplitThreads<NB, M, EN>::kAll) k_macro3(Params<R> p, InletTables<R> it, StepArgs<R> a,
+                                                                          R* aux) {
   using F = SplitFields<R, M, EN>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   after_previous();
-  const int lane = threadIdx.x % NB, l = group_of<NB>();
+  const int lane = threadIdx.x % NB, l = group_of<NB, M, EN>();
   R* S = reinterpret_cast<R*>(smem_raw) + lane;
   const int n = min((int)(blockIdx.x * NB) + lane, p.N - 1);
   {
@@ -358,16 +381,17 @@ __device__ __noinline__ void solve_row_fp64(const Params<R>& p, const R* S, R ph
 // (src: [M + 2][N] in double, mass production per species, then the change of
 // the fluid internal energy).
 template <class R, int M, bool EN, int NB, bool SRC, int MINB, bool PARK>
-__global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
+__global__ void __launch_bounds__(SplitThreads<NB, M, EN>::kAll, MINB)
     k_collide3(Params<R> p, InletTables<R> it, StepArgs<R> a, const double* srcv) {
   using F = SplitFields<R, M, EN>;
   constexpr int L = M + 1 + (EN ? 1 : 0);
+  constexpr int TS = SplitThreads<NB, M, EN>::kSp, T1 = SplitThreads<NB, M, EN>::kOne;
   // barriers: 0 all; 1 state ready (last group to the species), 2 pivot rows
   // (species), 3 mixture ready (last group to the momentum group), 4
   // difference moments (species), 5 v ready (species to the last group)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   after_previous();
-  const int lane = threadIdx.x % NB, l = group_of<NB>();
+  const int lane = threadIdx.x % NB, l = group_of<NB, M, EN>();
   R* S = reinterpret_cast<R*>(smem_raw) + lane;
   R* D0 = reinterpret_cast<R*>(smem_raw) + F::kAll * NB + lane * F::kStride;
   const bool live = (int)(blockIdx.x * NB) + lane < p.N;
@@ -439,7 +463,7 @@ __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
   };
   if (l < M) {
     // ---- species l: its row of the diffusion system (Eq. 23, 24, 22, 26, 29) ------
-    bar_sync(1, NB * (M + 1));
+    bar_sync(1, TS + T1);
     R w[3], v[3], row[M], X[M];
 #pragma unroll
     for (int b = 0; b < 3; ++b) w[b] = S[(F::kW + b) * NB];
@@ -486,7 +510,8 @@ __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
           pv[(M + b) * NB] = v[b];
         }
       }
-      bar_sync(2, NB * M);
+      if (NB < 32) __syncwarp();
+      bar_sync(2, TS);
       if (l != k) {
         const R g = row[k];
 #pragma unroll
@@ -512,7 +537,7 @@ __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
     }
 #pragma unroll
     for (int b = 0; b < 3; ++b) S[(F::kV + 3 * l + b) * NB] = v[b];
-    bar_arrive(5, NB * (M + 1));
+    bar_arrive(5, TS + T1);
     // ---- its difference moments and relaxation (Eq. 21, Eq. 25) --------------------
     const R gd = q * itk, qY = R(2) * q * hYl;         // (1 - beta) Y_l C
     SpeciesTarget<R, 3> t;
@@ -537,28 +562,28 @@ __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
       ax.template delta<2>(m);
       store16<9>(d + F::kO2, m);
     }
-    bar_sync(4, NB * M);
+    bar_sync(4, TS);
 #pragma unroll
     for (int b = 0; b < M; ++b) X[b] = (b == l) ? -gd : qY * p.invDmm[l][b];
     const R keep = R(1) - R(2) * beta;
-    R T2[9], T1[9], m[9], acc;
-    couple<R, M, F::kStride, NB, 9>(D0 + F::kO2, X, T2);
-    couple<R, M, F::kStride, NB, 9>(D0 + F::kO1, X, T1);
+    R c2[9], c1[9], m[9], acc;
+    couple<R, M, F::kStride, NB, 9>(D0 + F::kO2, X, c2);
+    couple<R, M, F::kStride, NB, 9>(D0 + F::kO1, X, c1);
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
-      T2[e] += t.template entry<2>(ax, w, e % 3, e / 3);
-      T1[e] += t.template entry<1>(ax, w, e % 3, e / 3);
+      c2[e] += t.template entry<2>(ax, w, e % 3, e / 3);
+      c1[e] += t.template entry<1>(ax, w, e % 3, e / 3);
     }
 #pragma unroll
-    for (int e = 0; e < 9; ++e) m[e] = T2[e] - T1[e];
+    for (int e = 0; e < 9; ++e) m[e] = c2[e] - c1[e];
     acc = relax_dirs<R, 3, false>(get, -1, keep, m, nullptr, put);
 #pragma unroll
-    for (int e = 0; e < 9; ++e) m[e] = T2[e] + T1[e];
+    for (int e = 0; e < 9; ++e) m[e] = c2[e] + c1[e];
     acc += relax_dirs<R, 3, false>(get, 1, keep, m, nullptr, put);
-    couple<R, M, F::kStride, NB, 8>(D0 + F::kO0, X, T1);
+    couple<R, M, F::kStride, NB, 8>(D0 + F::kO0, X, c1);
 #pragma unroll
     for (int e = 1; e < 9; ++e)
-      m[e] = (T1[e - 1] + t.template entry<0>(ax, w, e % 3, e / 3)) - R(2) * T2[e];
+      m[e] = (c1[e - 1] + t.template entry<0>(ax, w, e % 3, e / 3)) - R(2) * c2[e];
     acc += relax_dirs<R, 3, false>(get, 0, keep, m, nullptr, put);
     put(13, total - acc);
     return;
@@ -584,7 +609,7 @@ __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
     S[F::kKT * NB] = p.knudsen ? kT : R(0);
 #pragma unroll
     for (int k = 0; k < M; ++k) S[(F::kHY + k) * NB] = hC * s.Y[k];
-    bar_arrive(1, NB * (M + 1));
+    bar_arrive(1, TS + T1);
     if (live && bad_state(s, inv_phi)) flag(a.status, 1);
     Grad<R, 3, M, EN> gr;
     gr.divu = S[F::kU * NB] + S[(F::kU + 1) * NB] + S[(F::kU + 2) * NB];
@@ -598,7 +623,7 @@ __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
     }
     Mixture<R, 3> mix;
     mix.template scalars<M, EN>(p, s, inv_phi, gr.divu);
-    bar_sync(5, NB * (M + 1));
+    bar_sync(5, TS + T1);
     R v[M][3], vbar[3];
 #pragma unroll
     for (int k = 0; k < M; ++k)
@@ -619,7 +644,7 @@ __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
       S[F::kOm * NB] = mix.omega;
       S[F::kCf * NB] = cf;
       S[F::kTot * NB] = s.sf + sum_rd;                                                // Eq. 78
-      bar_arrive(3, 2 * NB);
+      bar_arrive(3, 2 * T1);
       // ---- energy (Eq. 43, Eq. 51, Eq. 54, Eq. 88) --------------------------------
       int e = F::kMo + 4;
 #pragma unroll
@@ -649,7 +674,7 @@ __global__ void __launch_bounds__(NB * (M + 1 + (EN ? 1 : 0)), MINB)
     }
   } else {
     // ---- momentum (Eq. 42, Eq. 44, Eq. 87) -----------------------------------------
-    bar_sync(3, 2 * NB);
+    bar_sync(3, 2 * T1);
     Axis<R> F3[3];
 #pragma unroll
     for (int b = 0; b < 3; ++b) F3[b].set(R(1), S[(F::kF + 2 * b) * NB], S[(F::kF + 2 * b + 1) * NB]);

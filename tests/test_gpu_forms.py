@@ -182,3 +182,18 @@ def test_split_2d_solves_in_double_above_the_bound(L, nx, ny):
 def test_split_2d_six_species(L):
     """Six species on a two-dimensional lattice, form 10 and the tiles."""
     check_forms(L, anode(19, 6, 1), range(10, 13))
+
+
+# FP64 blocks of 8 nodes (up to 608), of 16 (up to 4864) and of 32: below, at and
+# past a block and each line, species of one warp on different faces
+@pytest.mark.parametrize("shape", [(3, 1, 2), (4, 2, 3), (38, 4, 4), (29, 7, 3), (203, 3, 8), (32, 19, 8),
+                                   (139, 7, 5)])
+def test_small_blocks_3d(L, shape):
+    wl = anode(*shape)
+    o = oracle.Oracle(wl)
+    o.step(2)
+    g = L.Lattice(wl, precision=L.LBM_FP64)
+    g.step(2)
+    g.sync()
+    assert worst(g.populations(), o.pops()) < 1e-12
+    g.close()
