@@ -120,7 +120,7 @@ def other_forms(stream, torch, lbm):
         "note": "forward with checkpoints + recomputation + reverse sweep per step (wall clock)",
         "gradient_error_vs_fp64": float(np.max(np.abs(g32 - g64)) / np.max(np.abs(g64)))}
     # 3-D anode without reactions (D3Q27, six species, energy): 200 timed
-    # steps after 20 warm-up steps in the default form (staged two-pass), and
+    # steps after 20 warm-up steps in the default form (split by lattice), and
     # the plain FP64 step
     wl = W.anode3d()
     g = lbm.Lattice(wl, precision=lbm.LBM_FP32, stream=sp)
@@ -584,11 +584,10 @@ def profile_form(which):
     slab: the 512x512 slab in FP32, default form (TMA row march), 3 steps;
     slab_fp64: the same in FP64;
     slab2048: the 2048x2048 slab in FP32 (the back-to-back line), 3 steps;
-    anode: D3Q27 anode 64x32x32, six species, FP32, the default form (staged
-      with a gradient pass, variant 5), 3 steps; anode_gather: the staged form
-      that gathers its gradient inputs (variant 3);
+    anode: D3Q27 anode 64x32x32, six species, FP32, the default form (split by
+      lattice, variant 5), 3 steps; anode_gather: the same step as variant 3;
     react: the same lattice with the seeded surface mechanism, FP32, 3 steps;
-    batch: the 64-capillary sweep, FP32, staged persistent form (variant 7),
+    batch: the 64-capillary sweep, FP32, one block per 8 x 4 tile (variant 7),
       5 steps launched one by one (timing on, so no graph replay);
     adjoint: 64x64 adjoint slab, FP32, 10 steps with checkpoints every 5."""
     from paper_2409_02930_gb300 import lbm

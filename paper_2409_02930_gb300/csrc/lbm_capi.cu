@@ -217,6 +217,76 @@ void make_params(const lbm_config* c, Params<double>& p, InletTables<double>& it
 
 }  // namespace lbm
 
+// nu = A B: r species whose columns of nu are linearly independent (the basis,
+// those of the fewest steps first), A = nu restricted to them, B = every
+// species' change in terms of theirs.
+static void factor_stoichiometry(lbm::MechDev& h) {
+  const int NS = h.M + h.S, R = h.R;
+  std::vector<std::vector<double>> col(NS, std::vector<double>(R, 0.0));
+  std::vector<int> order(NS);
+  for (int a = 0; a < NS; ++a) {
+    order[a] = a;
+    for (int q = 0; q < h.nsr[a]; ++q) col[a][h.sr_k[a][q]] = h.sr_nud[a][q];
+  }
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return h.nsr[a] < h.nsr[b]; });
+  // eliminated columns of the basis: row piv of reduced[i] is 1 there and 0 in
+  // the other reduced columns; comb[i] expresses reduced[i] by the basis
+  std::vector<std::vector<double>> reduced, comb;
+  std::vector<int> piv;
+  h.r = 0;
+  for (int a : order) {
+    std::vector<double> v = col[a], w(NS, 0.0);
+    double top = 0.0;
+    for (double t : v) top = std::fmax(top, std::fabs(t));
+    for (size_t i = 0; i < reduced.size(); ++i) {
+      const double f = v[piv[i]];
+      if (f == 0.0) continue;
+      for (int k = 0; k < R; ++k) v[k] -= f * reduced[i][k];
+      for (int j = 0; j < NS; ++j) w[j] += f * comb[i][j];
+    }
+    int p = 0;
+    for (int k = 1; k < R; ++k)
+      if (std::fabs(v[k]) > std::fabs(v[p])) p = k;
+    if (std::fabs(v[p]) <= 1e-9 * top) {                 // dependent (or not taking part)
+      for (int j = 0; j < h.r; ++j)
+        if (std::fabs(w[j]) > 1e-12) {
+          h.bi[a][h.nb[a]] = j;
+          h.bv[a][h.nb[a]] = w[j];
+          h.bvf[a][h.nb[a]] = (float)w[j];
+          ++h.nb[a];
+        }
+      continue;
+    }
+    const double s = 1.0 / v[p];
+    for (double& t : v) t *= s;
+    for (double& t : w) t *= -s;
+    w[h.r] += s;
+    for (size_t i = 0; i < reduced.size(); ++i) {
+      const double f = reduced[i][p];
+      if (f == 0.0) continue;
+      for (int k = 0; k < R; ++k) reduced[i][k] -= f * v[k];
+      for (int j = 0; j < NS; ++j) comb[i][j] -= f * w[j];
+    }
+    reduced.push_back(v);
+    comb.push_back(w);
+    piv.push_back(p);
+    h.bas[h.r] = a;
+    h.bi[a][0] = h.r;
+    h.bv[a][0] = 1.0;
+    h.bvf[a][0] = 1.0f;
+    h.nb[a] = 1;
+    ++h.r;
+  }
+  for (int k = 0; k < R; ++k)
+    for (int i = 0; i < h.r; ++i)
+      if (col[h.bas[i]][k] != 0.0) {
+        h.ai[k][h.na[k]] = i;
+        h.avf[k][h.na[k]] = (float)col[h.bas[i]][k];
+        h.av[k][h.na[k]] = col[h.bas[i]][k];
+        ++h.na[k];
+      }
+}
+
 // Device state of a surface mechanism: coverages, per-node sources and the
 // mechanism table in SI units (the surface source works in FP64).
 static int setup_surface(lbm_ctx* x, const lbm_config* c) {
@@ -236,7 +306,6 @@ static int setup_surface(lbm_ctx* x, const lbm_config* c) {
         if (h.npart[k] >= 8) return fail(nullptr, LBM_ERR_ARG, "at most 8 species take part in one surface step");
         h.pidx[k][h.npart[k]] = a;
         h.pnu[k][h.npart[k]] = v;
-        h.pnuf[k][h.npart[k]] = (float)v;
         h.npart[k]++;
         h.sr_k[a][h.nsr[a]] = k;
         h.sr_nud[a][h.nsr[a]] = v;
@@ -260,6 +329,7 @@ static int setup_surface(lbm_ctx* x, const lbm_config* c) {
       for (int a = 0; a < c->M; ++a)
         if (c->nu_gas[k * c->M + a] != 0) return fail(nullptr, LBM_ERR_ARG, "a TPB step involves adsorbates only");
   }
+  factor_stoichiometry(h);
   if (c->edge) {
     h.l_tpb = c->l_tpb;
     h.beta_ct = c->beta_ct;

@@ -30,10 +30,18 @@ struct MechDev {
   int npart[RMAX];                   // species taking part in each step (nonzero stoichiometry)
   int pidx[RMAX][8];
   double pnu[RMAX][8];
-  float pnuf[RMAX][8];
   int nsr[MMAX + SMAX];               // steps in which each species takes part
   int sr_k[MMAX + SMAX][RMAX];
   double sr_nud[MMAX + SMAX][RMAX];
+  // nu = A B of rank r (A: the columns of r basis species, B: every species'
+  // change by theirs): entries of A per step, of B per species
+  int r, bas[MMAX + SMAX];
+  int na[RMAX], ai[RMAX][8];
+  double av[RMAX][8];
+  float avf[RMAX][8];
+  int nb[MMAX + SMAX], bi[MMAX + SMAX][MMAX + SMAX];
+  double bv[MMAX + SMAX][MMAX + SMAX];
+  float bvf[MMAX + SMAX][MMAX + SMAX];
   int nre[RMAX];                     // reactants of each step
   int ridx[RMAX][4];
   int rord[RMAX][4];
@@ -55,10 +63,13 @@ struct MechDev {
 
 constexpr double FARADAY_DEV = 96485.33212;   // C/mol
 
-// stoichiometric coefficient of the q-th species of step k, in the Jacobian's precision
-template <class RK> __device__ __forceinline__ RK pnu_of(const MechDev& mc, int k, int q);
-template <> __device__ __forceinline__ float pnu_of<float>(const MechDev& mc, int k, int q) { return mc.pnuf[k][q]; }
-template <> __device__ __forceinline__ double pnu_of<double>(const MechDev& mc, int k, int q) { return mc.pnu[k][q]; }
+// q-th entry of A of step k and of B of species j, in the Jacobian's precision
+template <class RK> __device__ __forceinline__ RK a_of(const MechDev& mc, int k, int q);
+template <> __device__ __forceinline__ float a_of<float>(const MechDev& mc, int k, int q) { return mc.avf[k][q]; }
+template <> __device__ __forceinline__ double a_of<double>(const MechDev& mc, int k, int q) { return mc.av[k][q]; }
+template <class RK> __device__ __forceinline__ RK b_of(const MechDev& mc, int j, int q);
+template <> __device__ __forceinline__ float b_of<float>(const MechDev& mc, int j, int q) { return mc.bvf[j][q]; }
+template <> __device__ __forceinline__ double b_of<double>(const MechDev& mc, int j, int q) { return mc.bv[j][q]; }
 
 __device__ __forceinline__ double ipow(double x, int n) {
   double r = 1.0;
@@ -72,9 +83,10 @@ __device__ __forceinline__ double ipow(double x, int n) {
 //
 // Mixed precision (iterative refinement): concentrations, rates, the
 // residual F = xi - dt r(xi) and the extents are FP64; the Newton systems are
-// solved in FP32 (RK = float) or FP64 (RK = double) through the species-space
-// matrix K = I - V U of the Woodbury identity (NS x NS instead of R x R),
-// whose factors are reused across iterations (simplified Newton) until the
+// solved in FP32 (RK = float) or FP64 (RK = double) in the space of the r
+// independent species changes (Woodbury identity, r x r instead of R x R: 9
+// for the 20 steps and 14 species of the anode mechanism), whose factors are
+// reused across iterations (simplified Newton) until the
 // contraction of the steps slows down or a step is shortened, when they are
 // rebuilt at the current iterate.  The FP64 residual fixes the root, so every variant
 // converges to the same FP64 solution.
@@ -88,7 +100,10 @@ __device__ __forceinline__ double ipow(double x, int n) {
 // over the pivots with the pivot row in registers and the triangular solves
 // over both indices with the right-hand side in registers, so each multiply-
 // add touches local memory once (twice while factorising) instead of twice
-// (three times).
+// (three times).  Solving in the r independent changes instead of all species'
+// (9 for 14 in the anode mechanism: 243 multiply-adds per factorisation for 915,
+// 0.3 KB of factors for 0.8) took the 128 x 64 x 64 FP32 reactive step from 4.42
+// to 3.55 ms; on the warp form, bound by its chain of steps, it changed nothing.
 template <int M, class RK>
 __device__ void surface_source_dev(const MechDev& mc, double T, const double* rho_a, double phi, const double* Xs0,
                                    double* rhodot, double* Xs1, double& dU, double& current, double dphi,
@@ -109,10 +124,11 @@ __device__ void surface_source_dev(const MechDev& mc, double T, const double* rh
   }
   const double scale = mc.a_s / phi;     // gas concentration change per extent
   const RK rscale = RK(scale);
-  // J = I - U V with U = dt dr/dc (R x NS, the reactants of each step) and
-  // V = diag(scale) nu^T (NS x R); by the Woodbury identity
-  // J^-1 b = b + U K^-1 V b with K = I - V U (NS x NS), whose LU factors and U
-  // are kept while the iteration reuses them.
+  // J = I - U diag(scale) B^T A^T with U = dt dr/dc (R x NS, the reactants of
+  // each step); by the Woodbury identity J^-1 b = b + U z, z = diag(scale) B^T y,
+  // K y = A^T b with K = I - A^T U diag(scale) B^T (r x r, the determinant of J),
+  // whose LU factors and U are kept while the iteration reuses them.
+  const int r_ = mc.r;
   RK LU[NSX][NSX];
   RK uk[RMAX][4];
   int perm[NSX];
@@ -124,11 +140,11 @@ __device__ void surface_source_dev(const MechDev& mc, double T, const double* rh
     for (int i = 0; i < NS; ++i) {
       c[i] = c0[i] + (i < M ? scale : 1.0) * d[i];
       pos[i] = fmax(c[i], 0.0);
-      w[i] = RK(0);
     }
+    for (int i = 0; i < r_; ++i) w[i] = RK(0);
     if (refresh)
-      for (int i = 0; i < NS; ++i)
-        for (int j = 0; j < NS; ++j) LU[i][j] = (i == j) ? RK(1) : RK(0);
+      for (int i = 0; i < r_; ++i)
+        for (int j = 0; j < r_; ++j) LU[i][j] = (i == j) ? RK(1) : RK(0);
     for (int k = 0; k < Rn; ++k) {
       // rate r = k prod c^o; where the Jacobian is rebuilt also its derivatives
       // u_j = dt k o_j c_j^(o_j - 1) prod of the others (zero where c_j <= 0)
@@ -149,10 +165,8 @@ __device__ void surface_source_dev(const MechDev& mc, double T, const double* rh
       if (nre > 2) r *= f[2] * f[3];
       const RK bk = RK(-(xi[k] - mc.dt * r));
       b[k] = bk;
-      for (int q = 0; q < mc.npart[k]; ++q) {
-        const int i = mc.pidx[k][q];
-        w[i] += (i < M ? rscale : RK(1)) * pnu_of<RK>(mc, k, q) * bk;
-      }
+      const int na = mc.na[k];
+      for (int q = 0; q < na; ++q) w[mc.ai[k][q]] += a_of<RK>(mc, k, q) * bk;
       if (refresh) {
         const double dk = mc.dt * kr[k];
 #pragma unroll
@@ -164,23 +178,26 @@ __device__ void surface_source_dev(const MechDev& mc, double T, const double* rh
           for (int e = 0; e < 4; ++e)
             if (e != j && e < nre) u *= f[e];
           const RK ur = c[jj] > 0.0 ? RK(u * mc.rord[k][j]) : RK(0);
-          uk[k][j] = ur;
-          for (int q = 0; q < mc.npart[k]; ++q) {
-            const int i = mc.pidx[k][q];
-            LU[i][jj] -= (i < M ? rscale : RK(1)) * pnu_of<RK>(mc, k, q) * ur;
+          const RK us = jj < M ? rscale * ur : ur;
+          uk[k][j] = us;
+          const int nb = mc.nb[jj];
+          for (int e = 0; e < nb; ++e) {
+            const RK t = us * b_of<RK>(mc, jj, e);
+            const int i2 = mc.bi[jj][e];
+            for (int q = 0; q < na; ++q) LU[mc.ai[k][q]][i2] -= a_of<RK>(mc, k, q) * t;
           }
         }
       }
     }
     if (refresh) {
       // LU factors of K with partial pivoting (row order recorded in perm)
-      for (int i = 0; i < NS; ++i) perm[i] = i;
+      for (int i = 0; i < r_; ++i) perm[i] = i;
 #pragma unroll
       for (int cc = 0; cc < NSX; ++cc) {
-        if (cc >= NS) break;
+        if (cc >= r_) break;
         int pv = cc;
         RK best = fabs(LU[cc][cc]);
-        for (int k = cc + 1; k < NS; ++k) {
+        for (int k = cc + 1; k < r_; ++k) {
           const RK v = fabs(LU[k][cc]);
           if (v > best) {
             best = v;
@@ -193,7 +210,7 @@ __device__ void surface_source_dev(const MechDev& mc, double T, const double* rh
         perm[cc] = pp;
 #pragma unroll
         for (int l = 0; l < NSX; ++l) {
-          if (l >= NS) break;
+          if (l >= r_) break;
           const RK t = LU[cc][l];
           prow[l] = LU[pv][l];
           if (pv != cc) {
@@ -202,12 +219,12 @@ __device__ void surface_source_dev(const MechDev& mc, double T, const double* rh
           }
         }
         const RK inv = RK(1) / prow[cc];
-        for (int k = cc + 1; k < NS; ++k) {
+        for (int k = cc + 1; k < r_; ++k) {
           const RK f = LU[k][cc] * inv;
           LU[k][cc] = f;
 #pragma unroll
           for (int l = cc + 1; l < NSX; ++l) {
-            if (l >= NS) break;
+            if (l >= r_) break;
             LU[k][l] -= f * prow[l];
           }
         }
@@ -215,33 +232,40 @@ __device__ void surface_source_dev(const MechDev& mc, double T, const double* rh
       }
       refresh = false;
     }
-    // solve J dxi = -F:  w = V b, K z = w, dxi = b + U z
+    // solve J dxi = -F:  w = A^T b, K y = w, z = B^T y (U holds the scale), dxi = b + U z
+    RK z[NSX];
     {
       RK y[NSX];
 #pragma unroll
       for (int k = 0; k < NSX; ++k) {
-        if (k >= NS) break;
+        if (k >= r_) break;
         y[k] = w[perm[k]];
 #pragma unroll
         for (int l = 0; l < k; ++l) y[k] -= LU[k][l] * y[l];
       }
 #pragma unroll
       for (int k = NSX - 1; k >= 0; --k) {
-        if (k >= NS) continue;
+        if (k >= r_) continue;
 #pragma unroll
         for (int l = k + 1; l < NSX; ++l) {
-          if (l >= NS) break;
+          if (l >= r_) break;
           y[k] -= LU[k][l] * y[l];
         }
         y[k] *= LU[k][k];
         w[k] = y[k];
       }
     }
+    for (int i = 0; i < NS; ++i) {
+      RK t = RK(0);
+      const int nb = mc.nb[i];
+      for (int e = 0; e < nb; ++e) t += b_of<RK>(mc, i, e) * w[mc.bi[i][e]];
+      z[i] = t;
+    }
     double dd[NSX], dxi[RMAX];
     for (int i = 0; i < NS; ++i) dd[i] = 0.0;
     for (int k = 0; k < Rn; ++k) {
       RK x = b[k];
-      for (int j = 0; j < mc.nre[k]; ++j) x += uk[k][j] * w[mc.ridx[k][j]];
+      for (int j = 0; j < mc.nre[k]; ++j) x += uk[k][j] * z[mc.ridx[k][j]];
       dxi[k] = (double)x;
       for (int j = 0; j < mc.npart[k]; ++j) dd[mc.pidx[k][j]] += mc.pnu[k][j] * dxi[k];
     }
@@ -326,8 +350,8 @@ __global__ void __launch_bounds__(128, MINB) k_source(int N, const R* aux, const
 }
 
 // Which form a lattice of N nodes takes.  A warp per node up to 2048 nodes
-// (FP64 12 x 2 x 2: 157 us per reactive step against 380 us with a thread per
-// node; 8192 nodes FP32 376 against 303, so the line lies below 152 SMs x a few
+// (measured before the solve in r changes, FP64 12 x 2 x 2: 157 us per reactive
+// step against 380 us with a thread per node; 8192 nodes FP32 376 against 303, so the line lies below 152 SMs x a few
 // warps).  Above it a thread per node: without a register limit while the
 // threads do not fill the GPU (8192 nodes FP32 303 us per step at 222
 // registers, 332 at 48), then limited to 48 (FP32) or 64 (FP64) registers, so
@@ -340,7 +364,7 @@ constexpr int source_wide_nodes = 152 * 128 * 2;
 // GPU with a thread per node: there the time is the latency of one node's
 // Newton iteration, whose loops a warp runs side by side.  Lane k holds
 // reaction k (rate, extent, Jacobian entries), lane i species i
-// (concentration, row i of K in registers); rows are eliminated in pivot
+// (concentration) and row i of K in registers; rows are eliminated in pivot
 // order without being moved (the pivot lane's row is broadcast by shuffles),
 // so no work array is indexed dynamically.  The iteration, its thresholds and
 // the precision of every quantity are those of surface_source_dev; sums run
@@ -353,16 +377,26 @@ __global__ void __launch_bounds__(32) k_source_warp(int N, const RK* aux, const 
   constexpr unsigned FULL = 0xffffffffu;
   __shared__ double s_nu[RMAX][NSX], s_c[32], s_x[32];
   __shared__ unsigned char s_k[RMAX][NSX];
-  __shared__ RK s_b[32], s_u[RMAX][4], s_K[NSX][NSX + 1];
+  __shared__ RK s_b[32], s_u[RMAX][4], s_K[NSX][NSX + 1], s_y[32], s_bv[NSX][NSX];
+  __shared__ unsigned char s_bi[NSX][NSX], s_nb[32];
   const int lane = threadIdx.x;
   const MechDev& mc = *ra.mech;
-  const int S = mc.S, Rn = mc.R, NS = M + S;
+  const int S = mc.S, Rn = mc.R, NS = M + S, r_ = mc.r;
   const bool sp = lane < NS, re = lane < Rn;
   const int nq = sp ? mc.nsr[lane] : 0;
   for (int q = 0; q < nq; ++q) {
     s_k[q][lane] = (unsigned char)mc.sr_k[lane][q];
     s_nu[q][lane] = mc.sr_nud[lane][q];
   }
+  // B of species `lane`, and the basis species of row `lane` of K
+  const int nb = sp ? mc.nb[lane] : 0;
+  for (int e = 0; e < nb; ++e) {
+    s_bi[e][lane] = (unsigned char)mc.bi[lane][e];
+    s_bv[e][lane] = b_of<RK>(mc, lane, e);
+  }
+  s_nb[lane] = (unsigned char)nb;
+  const bool rowl = lane < r_;
+  const int bs = rowl ? mc.bas[lane] : 0, nqb = rowl ? mc.nsr[bs] : 0;
   int nre = 0, ri[4], ro[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) ri[j] = ro[j] = 0;
@@ -380,6 +414,7 @@ __global__ void __launch_bounds__(32) k_source_warp(int N, const RK* aux, const 
   const double ph = (double)phi[n], T = (double)aux[(size_t)M * N + n];
   const double dphi = mc.dphi_field ? mc.dphi_field[n] : mc.dphi;
   const double scale = lane < M ? mc.a_s / ph : 1.0;       // concentration change per extent of species `lane`
+  const RK gscale = RK(mc.a_s / ph);
   double c0 = 0.0, Xs0 = 0.0;
   if (lane < M) c0 = (double)(aux[(size_t)lane * N + n] / phi[n]) / mc.m[lane];
   else if (sp) {
@@ -414,32 +449,36 @@ __global__ void __launch_bounds__(32) k_source_warp(int N, const RK* aux, const 
       for (int j = 0; j < 4; ++j) {
         if (j < nre) {
           const double cj = s_c[ri[j]];
-          uk[j] = cj > 0.0 ? RK(mc.dt * r * ro[j] / cj) : RK(0);
+          uk[j] = cj > 0.0 ? RK(mc.dt * r * ro[j] / cj) * (ri[j] < M ? gscale : RK(1)) : RK(0);
         }
         s_u[lane][j] = uk[j];
       }
     }
     __syncwarp();
     if (refresh) {
-      // row `lane` of K = I - V U
-      if (sp) {
-        for (int j = 0; j < NS; ++j) s_K[lane][j] = (j == lane) ? RK(1) : RK(0);
-        for (int q = 0; q < nq; ++q) {
-          const int k = s_k[q][lane];
-          const RK v = RK(scale * s_nu[q][lane]);
+      // row `lane` of K = I - A^T U diag(scale) B^T
+      if (rowl) {
+        for (int j = 0; j < r_; ++j) s_K[lane][j] = (j == lane) ? RK(1) : RK(0);
+        for (int q = 0; q < nqb; ++q) {
+          const int k = s_k[q][bs];
+          const RK v = RK(s_nu[q][bs]);
           const int m = mc.nre[k];
-          for (int j = 0; j < m; ++j) s_K[lane][mc.ridx[k][j]] -= v * s_u[k][j];
+          for (int j = 0; j < m; ++j) {
+            const int jj = mc.ridx[k][j];
+            const RK t = v * s_u[k][j];
+            for (int e = 0; e < s_nb[jj]; ++e) s_K[lane][s_bi[e][jj]] -= t * s_bv[e][jj];
+          }
         }
       }
 #pragma unroll
-      for (int j = 0; j < NSX; ++j) row[j] = (sp && j < NS) ? s_K[lane][j] : RK(0);
+      for (int j = 0; j < NSX; ++j) row[j] = (rowl && j < r_) ? s_K[lane][j] : RK(0);
       // LU with partial pivoting: the largest entry of the column among the
       // rows not yet taken (compared in single precision, lane in the low bits)
-      bool taken = !sp;
+      bool taken = !rowl;
       mine = NSX;
 #pragma unroll
       for (int cc = 0; cc < NSX; ++cc) {
-        if (cc >= NS) break;
+        if (cc >= r_) break;
         const unsigned bits = (__float_as_uint((float)fabs(row[cc])) & ~31u) | 32u;
         const unsigned key = taken ? 0u : (bits | (unsigned)lane);
         pl[cc] = (int)(__reduce_max_sync(FULL, key) & 31u);
@@ -451,7 +490,7 @@ __global__ void __launch_bounds__(32) k_source_warp(int N, const RK* aux, const 
         const RK f = row[cc] * inv[cc];
 #pragma unroll
         for (int j = cc + 1; j < NSX; ++j) {
-          if (j >= NS) break;
+          if (j >= r_) break;
           const RK pj = __shfl_sync(FULL, row[j], pl[cc]);
           if (!taken) row[j] -= f * pj;
         }
@@ -459,23 +498,27 @@ __global__ void __launch_bounds__(32) k_source_warp(int N, const RK* aux, const 
       }
       refresh = false;
     }
-    // solve J dxi = -F:  w = V b, K z = w, dxi = b + U z
+    // solve J dxi = -F:  w = A^T b, K y = w, z = B^T y (U holds the scale), dxi = b + U z
     RK w = RK(0);
-    for (int q = 0; q < nq; ++q) w += RK(scale * s_nu[q][lane]) * s_b[s_k[q][lane]];
+    for (int q = 0; q < nqb; ++q) w += RK(s_nu[q][bs]) * s_b[s_k[q][bs]];
 #pragma unroll
     for (int cc = 0; cc < NSX; ++cc) {
-      if (cc >= NS) break;
+      if (cc >= r_) break;
       const RK wp = __shfl_sync(FULL, w, pl[cc]);
-      if (sp && mine > cc) w -= row[cc] * wp;
+      if (rowl && mine > cc) w -= row[cc] * wp;
     }
-    RK z = RK(0);
+    RK y = RK(0);
 #pragma unroll
     for (int cc = NSX - 1; cc >= 0; --cc) {
-      if (cc >= NS) continue;
+      if (cc >= r_) continue;
       const RK xc = __shfl_sync(FULL, w, pl[cc]) * inv[cc];
-      if (sp && mine < cc) w -= row[cc] * xc;
-      if (lane == cc) z = xc;
+      if (rowl && mine < cc) w -= row[cc] * xc;
+      if (lane == cc) y = xc;
     }
+    s_y[lane] = y;
+    __syncwarp();
+    RK z = RK(0);
+    for (int e = 0; e < nb; ++e) z += s_bv[e][lane] * s_y[s_bi[e][lane]];
     double dxi = 0.0;
     {
       RK x = b;

@@ -1,9 +1,8 @@
 // Two-pass form of the step, and the macroscopic fields for lbm_moments.
 //
 // 2-D nodes hold their 5 x 9 (or fewer) streamed populations in registers
-// (pull_node: every load independent and in flight at once); a D3Q27 node's
-// array is too large for that and lives in local memory, where the staged
-// forms (lbm_staged.cuh) are used instead.
+// (pull_node: every load independent and in flight at once).  D3Q27 steps run
+// split by lattice (lbm_split3d.cuh); here they only take their moments.
 #pragma once
 
 #include "lbm_compact.cuh"

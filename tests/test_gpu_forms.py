@@ -197,3 +197,23 @@ def test_small_blocks_3d(L, shape):
     g.sync()
     assert worst(g.populations(), o.pops()) < 1e-12
     g.close()
+
+
+@pytest.mark.parametrize("steps", [1, 2, 7])
+def test_surface_source_of_low_rank_mechanisms(L, steps):
+    """The first steps of the mechanism only: one independent change, a step and
+    its reverse, and species that take no part; a warp and a thread per node."""
+    mc = W.surface_mechanism()
+    for k in ("nu_gas", "nu_surf", "A", "Ea"):
+        setattr(mc, k, np.ascontiguousarray(getattr(mc, k)[:steps]))
+    mc.R = steps
+    for shape in ((4, 2, 2), (17, 11, 11)):
+        wl = W.anode3d(*shape, mechanism=mc, steps=2)
+        o = oracle.Oracle(wl)
+        o.step(2)
+        g = L.Lattice(wl, precision=L.LBM_FP64)
+        g.step(2)
+        g.sync()
+        assert worst(g.populations(), o.pops()) < 1e-12
+        assert np.max(np.abs(g.moments(L.LBM_MOM_XS) - o.moments(oracle.MOM_XS))) < 1e-12
+        g.close()
