@@ -331,8 +331,9 @@ int lbm_get_timing(lbm_ctx* ctx, double* ms_by_kind /* [3] */, long long* launch
  * default).  Every form
  * computes the same step (the gradient stencil is summed in different
  * orders, so the forms agree to rounding).  New contexts use variant 5 in
- * 3-D and, in 2-D, variant 8 on FP32 lattices of at least 2^18 nodes with nx a
- * multiple of 4 and no reservoir face, else tiles (10 up to 9728 nodes, above
+ * 3-D and, in 2-D, variant 8 on FP32 lattices with nx a multiple of 4 and no
+ * reservoir face of at least 3 * 2^20 nodes, or of at least 2^18 in at most 1216
+ * blocks of 30 x 8 nodes, else tiles (10 up to 9728 nodes, above
  * that 12 in FP32 and 11 in FP64; lattices of one or two rows with 8192 nodes
  * or more: the two-pass form); batches use variant 10.  The adjoint's
  * forward and recompute steps use the context's form.  lbm_autotune times

@@ -71,26 +71,29 @@ void convert_inlet(const lbm::InletTables<double>& d, lbm::InletTables<R>& r) {
 constexpr int kDefaultWaitLimit = 1 << 22;
 
 // Kernel form of a new single lattice.  3-D: the split step.  2-D, measured in
-// us per step (tiles / row march / two-pass):
-//   FP32 256x256 with reservoirs 14.4 / 73 / 18.5, 512x512 30.8 / 30.9 / 43.7,
-//   701x523 with walls 45 / 58 / 70, 2048x2048 393 / 382 / 697;
-//   FP64 512x512 549 / 689 / 608.
+// us per step (tiles / row march): FP32 256x256 with reservoirs 14.4 / 73,
+//   512x512 28.0 / 28.0, 640x512 36.1 / 52.5, 512x768 43.0 / 54.5, 1024x512
+//   55.3 / 56.5, 1024x1024 104.6 / 108.4, 1536x1536 224 / 226, 2048x2048 389 /
+//   380, 701x523 with walls 45 / 58; FP64 512x512 549 / 689.
 // The row march (bulk tensor copies, rows of whole 16-byte units, no
-// reservoir) is taken from 2^18 FP32 nodes, where its prefetched rows read
-// HBM without stalls; everything else runs on tiles.  Up to two 32-node tiles
-// per SM the lattice is bound by one tile's latency and the tiles are split by
+// reservoir) is taken from 3 x 2^20 FP32 nodes, where its prefetched rows read
+// HBM without stalls, and from 2^18 nodes where its blocks (30 columns by 8
+// rows, eight resident per SM) make one wave, which they fill; between the two
+// its long blocks leave part of a last wave empty, and the tiles win.
+// Everything else runs on tiles.  Up to two 32-node tiles per SM the lattice is bound by one tile's latency and the tiles are split by
 // lattice (split / best other tile: FP64 256x4 20.0 / 40.1, capillary 17.5 /
 // 34.1, 96x96 27.5 / 40.4, 128x128 52.2 / 44.0; FP32 64x40 4.9 / 5.5, 96x96
 // 5.1 / 6.5, 128x128 7.4 / 6.0); above that 32 x 4 in FP32 (whole lines) and
 // 16 x 8 in FP64 (bound by operations, so the smaller halo counts).  Lattices
 // of one or two rows would leave most of a tile idle and take the two-pass
 // form once they fill the GPU.
-constexpr long long kSplit2dNodes = 2 * 152 * 32;
+constexpr long long kSplit2dNodes = 2 * 152 * 32, kMarchNodes = 3 << 20;
 int default_variant(const lbm_config* c) {
   if (c->nz > 1) return 5;
   const long long N = (long long)c->nx * c->ny;
   const bool reservoir = c->bc_lo == LBM_BC_INLET || c->bc_hi == LBM_BC_INLET;
-  if (c->precision == LBM_FP32 && !reservoir && N >= (1 << 18) && c->nx % 4 == 0) return 8;
+  const bool one_wave = N >= (1 << 18) && ((c->nx + 29LL) / 30) * ((c->ny + 7LL) / 8) <= 8 * 152;
+  if (c->precision == LBM_FP32 && !reservoir && (one_wave || N >= kMarchNodes) && c->nx % 4 == 0) return 8;
   if (c->ny > 4 * 65535 || (c->ny < 3 && N >= 8192)) return -1;
   return N <= kSplit2dNodes ? 10 : (c->precision == LBM_FP32 ? 12 : 11);
 }
