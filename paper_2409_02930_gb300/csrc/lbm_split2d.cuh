@@ -144,7 +144,6 @@ __global__ void __launch_bounds__(32 * (M + 2 + (EN ? 1 : 0))) k_split2d(Params<
         macro_fields<R, 2, M, EN>(s, [&](int k, const R& v) { m[k * PN] = v; });
       }
     }
-    __syncwarp();
     bar_sync(3, 64);
     // neighbours' rows inside the tile; cells beyond a ragged edge are computed
     // from whatever the tile holds and never stored

@@ -92,9 +92,19 @@ __device__ __forceinline__ int group_of() {
   return t < B::kSp ? min(t / NB, M - 1) : M + (t - B::kSp) / B::kOne;
 }
 
-// named barriers among `n` threads of the block
-__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(n) : "memory"); }
+// Named barriers among `n` threads of the block, whole warps.  A warp may come
+// here from branches that only some of its lanes took (reservoir and wall
+// columns, the FP64 solve, a flag), so it reconverges first, and the forms are
+// those that do not ask for a converged warp (bar.* is the aligned form, which
+// a warp that arrives in parts would be counted at more than once).
+__device__ __forceinline__ void bar_sync(int id, int n) {
+  __syncwarp();
+  asm volatile("barrier.cta.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+  __syncwarp();
+  asm volatile("barrier.cta.arrive %0, %1;\n" ::"r"(id), "r"(n) : "memory");
+}
 
 // two values as one register pair: FP32 pairs use the packed multiply-add
 template <class R> struct Pair;
@@ -510,7 +520,6 @@ __global__ void __launch_bounds__(SplitThreads<NB, M, EN>::kAll, MINB)
           pv[(M + b) * NB] = v[b];
         }
       }
-      if (NB < 32) __syncwarp();
       bar_sync(2, TS);
       if (l != k) {
         const R g = row[k];
