@@ -1,0 +1,44 @@
+// Which kernel form a new single lattice takes, from its configuration alone
+// (host code without CUDA).
+#pragma once
+
+#include "../../include/lbm.h"
+
+namespace lbm {
+
+// Forms whose grid counts rows in its y dimension can launch up to this many
+// units of `rows` lattice rows; taller lattices take a form with a flat grid.
+constexpr int kGridRows = 65535;
+inline bool rows_fit(long long ny, int rows) { return (ny + rows - 1) / rows <= kGridRows; }
+
+// Kernel form of a new single lattice.  3-D: the split step.  2-D, measured in
+// us per step (tiles / row march): FP32 256x256 with reservoirs 14.4 / 73,
+//   512x512 28.0 / 28.0, 640x512 36.1 / 52.5, 512x768 43.0 / 54.5, 1024x512
+//   55.3 / 56.5, 1024x1024 104.6 / 108.4, 1536x1536 224 / 226, 2048x2048 389 /
+//   380, 701x523 with walls 45 / 58; FP64 512x512 549 / 689.
+// The row march (bulk tensor copies, rows of whole 16-byte units, no
+// reservoir) is taken from 3 x 2^20 FP32 nodes, where its prefetched rows read
+// HBM without stalls, and from 2^18 nodes where its blocks (30 columns by 8
+// rows, eight resident per SM) make one wave, which they fill; between the two
+// its long blocks leave part of a last wave empty, and the tiles win.
+// Everything else runs on tiles.  Up to two 32-node tiles per SM the lattice is
+// bound by one tile's latency and the tiles are split by lattice (split / best other tile: FP64 256x4 20.0 / 40.1, capillary 17.5 /
+// 34.1, 96x96 27.5 / 40.4, 128x128 52.2 / 44.0; FP32 64x40 4.9 / 5.5, 96x96
+// 5.1 / 6.5, 128x128 7.4 / 6.0); above that 32 x 4 in FP32 (whole lines) and
+// 16 x 8 in FP64 (bound by operations, so the smaller halo counts).  Lattices
+// of one or two rows would leave most of a tile idle and take the two-pass
+// form once they fill the GPU, and so do lattices with more rows than the tiles'
+// grids can count.
+constexpr long long kSplit2dNodes = 2 * 152 * 32, kMarchNodes = 3 << 20;
+inline int default_variant(const lbm_config* c) {
+  if (c->nz > 1) return 5;
+  const long long N = (long long)c->nx * c->ny;
+  const bool reservoir = c->bc_lo == LBM_BC_INLET || c->bc_hi == LBM_BC_INLET;
+  const bool one_wave = N >= (1 << 18) && ((c->nx + 29LL) / 30) * ((c->ny + 7LL) / 8) <= 8 * 152;
+  if (c->precision == LBM_FP32 && !reservoir && (one_wave || N >= kMarchNodes) && c->nx % 4 == 0 && rows_fit(c->ny, 8))
+    return 8;
+  if (!rows_fit(c->ny, 4) || (c->ny < 3 && N >= 8192)) return -1;
+  return N <= kSplit2dNodes ? 10 : (c->precision == LBM_FP32 ? 12 : 11);
+}
+
+}  // namespace lbm

@@ -1,5 +1,6 @@
 // Instantiates the step kernels for one (precision, dimension); the including
 // file defines LBM_REAL, LBM_DIM and LBM_OPS_NAME.
+#include "lbm_forms.h"
 #include "lbm_fused.cuh"
 #include "lbm_march2d.cuh"
 #include "lbm_ops.h"
@@ -35,10 +36,10 @@ struct Launch {
   static int macro3(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, R* aux, cudaStream_t s) {
     if constexpr (D == 3) {
       constexpr size_t smem = split_smem_bytes<R, M, EN>(NB, false, false);
-      launch_after(k_macro3<R, M, EN, NB, AUX>, (p.N + NB - 1) / NB, SplitThreads<NB, M, EN>::kAll, smem, s, p, it, a,
-                   aux);
+      return launch_after(k_macro3<R, M, EN, NB, AUX>, (p.N + NB - 1) / NB, SplitThreads<NB, M, EN>::kAll, smem, s, p,
+                          it, a, aux);
     }
-    return 0;
+    return -1;
   }
   template <bool SRC, int NB, int MINB, bool PARK>
   static int collide3(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, const double* src,
@@ -48,9 +49,9 @@ struct Launch {
       auto kern = k_collide3<R, M, EN, NB, SRC, MINB, PARK>;
       static bool done = false;
       if (configure(kern, smem, done)) return -1;
-      launch_after(kern, (p.N + NB - 1) / NB, SplitThreads<NB, M, EN>::kAll, smem, s, p, it, a, src);
+      return launch_after(kern, (p.N + NB - 1) / NB, SplitThreads<NB, M, EN>::kAll, smem, s, p, it, a, src);
     }
-    return 0;
+    return -1;
   }
   static constexpr int kMinB = 2;
   static constexpr bool kPark = sizeof(R) == 4;
@@ -83,6 +84,7 @@ struct Launch {
   template <int TX, int TY, int SEG>
   static int fused_tile(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
     static_assert(D == 2, "fused tiles are a 2-D form");
+    if (!rows_fit(p.ny, SEG)) return -1;
     constexpr size_t smem = fused_smem_bytes<R, D, M, EN, TX, TY>();
     auto kern = k_fused<R, D, M, EN, TX, TY, SEG>;
     static bool done = false;
@@ -95,18 +97,18 @@ struct Launch {
   // tiles with the populations in registers
   template <int TX, int TY, int MINB>
   static int tile2d(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
-    if ((p.ny + TY - 1) / TY > 65535) return -1;
+    if (!rows_fit(p.ny, TY)) return -1;
     if constexpr (D == 2)
-      launch_after(k_tile2d<R, M, EN, TX, TY, MINB>, dim3((p.nx + TX - 1) / TX, (p.ny + TY - 1) / TY), TX * TY, 0, s, p,
-                   it, a);
-    return 0;
+      return launch_after(k_tile2d<R, M, EN, TX, TY, MINB>, dim3((p.nx + TX - 1) / TX, (p.ny + TY - 1) / TY), TX * TY,
+                          0, s, p, it, a);
+    return -1;
   }
   // tiles split by lattice, one warp each
   static int split2d(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
-    if ((p.ny + 3) / 4 > 65535) return -1;
+    if (!rows_fit(p.ny, 4)) return -1;
     if constexpr (D == 2)
-      launch_after(k_split2d<R, M, EN>, dim3((p.nx + 7) / 8, (p.ny + 3) / 4), 32 * (L + 1), 0, s, p, it, a);
-    return 0;
+      return launch_after(k_split2d<R, M, EN>, dim3((p.nx + 7) / 8, (p.ny + 3) / 4), 32 * (L + 1), 0, s, p, it, a);
+    return -1;
   }
   // pipelined 2-D step (cp.async staging), TX columns marching SEG rows
   template <int TX, int SEG, int MINB, int PD>
@@ -118,14 +120,14 @@ struct Launch {
       if constexpr (smem > kMaxSmem) {
         return -1;
       } else {
+        if (!rows_fit(p.ny, SEG)) return -1;
         // the reservoir-column path is compiled in only when a face is a reservoir
         const bool inlet = p.bc_lo == BC_INLET || p.bc_hi == BC_INLET;
         auto kern = inlet ? k_march2d<R, M, EN, TX, SEG, MINB, PD, true> : k_march2d<R, M, EN, TX, SEG, MINB, PD, false>;
         static bool done[2] = {false, false};
         if (configure(kern, smem, done[inlet ? 1 : 0])) return -1;
         dim3 g((p.nx + TX - 3) / (TX - 2), (p.ny + SEG - 1) / SEG, 1);
-        launch_after(kern, g, TX, smem, s, p, it, a, TmaMaps{});
-        return 0;
+        return launch_after(kern, g, TX, smem, s, p, it, a, TmaMaps{});
       }
     }
   }
@@ -141,6 +143,7 @@ struct Launch {
       if constexpr (smem > kMaxSmem) {
         return -1;
       } else {
+        if (!rows_fit(p.ny, SEG)) return -1;
         TmaMaps tm;
         if (!encode_row_maps<R>(tm, a.src, a.phi, EN ? nullptr : a.Tfix, p.nx, p.ny, Lat<D>::Q, LB::NL, LB::W))
           return march2d<TX, SEG, MINB, PD>(p, it, a, s);
@@ -150,8 +153,7 @@ struct Launch {
         static bool done[2] = {false, false};
         if (configure(kern, smem, done[inlet ? 1 : 0])) return -1;
         dim3 g((p.nx + TX - 3) / (TX - 2), (p.ny + SEG - 1) / SEG, 1);
-        launch_after(kern, g, TX, smem, s, p, it, a, tm);
-        return 0;
+        return launch_after(kern, g, TX, smem, s, p, it, a, tm);
       }
     }
   }
@@ -190,8 +192,7 @@ struct Launch {
         default: return -1;
       }
     } else {
-      if (v < 3) macro3<false, 32>(p, it, a, nullptr, s);
-      else macro_any<false>(p, it, a, nullptr, s);
+      if (v < 3 ? macro3<false, 32>(p, it, a, nullptr, s) : macro_any<false>(p, it, a, nullptr, s)) return -1;
       switch (v) {
         case 0: return collide3<false, 32, 1, false>(p, it, a, nullptr, s);
         case 1: return collide3<false, 32, 2, false>(p, it, a, nullptr, s);

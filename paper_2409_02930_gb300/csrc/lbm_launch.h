@@ -25,8 +25,10 @@
 
 namespace lbm {
 
+// Returns 0, or -1 where the launch was refused (the error also stays with
+// cudaGetLastError for callers that launch several kernels).
 template <class... K, class... A>
-inline void launch_after(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+inline int launch_after(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
@@ -37,7 +39,7 @@ inline void launch_after(void (*kern)(K...), dim3 grid, dim3 block, size_t smem,
   c.stream = s;
   c.attrs = &at;
   c.numAttrs = 1;
-  cudaLaunchKernelEx(&c, kern, std::forward<A>(args)...);   // errors surface through cudaGetLastError
+  return cudaLaunchKernelEx(&c, kern, std::forward<A>(args)...) == cudaSuccess ? 0 : -1;
 }
 
 #ifdef __CUDACC__
