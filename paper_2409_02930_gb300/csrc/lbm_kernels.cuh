@@ -10,11 +10,11 @@ namespace lbm {
 // Arguments shared by the step kernels (device pointers).
 template <class R>
 struct StepArgs {
-  const R* __restrict__ src;     // post-collision populations of the previous step
-  R* __restrict__ dst;           // new post-collision populations
+  const R* src;                  // post-collision populations of the previous step
+  R* dst;                        // new post-collision populations
   const R* __restrict__ phi;     // porosity [N]
   const R* __restrict__ Tfix;    // fixed temperature [N] (isothermal lattices)
-  R* __restrict__ mac;           // macro fields for the gradients [2D+M][N]
+  R* mac;                        // macro fields for the gradients [2D+M][N]
   int* status;                   // bit 0: non-finite / non-positive density, bit 1: FP64 solve used,
                                  // bit 2: surface Newton not converged, bit 3: a bounded wait gave up
 };

@@ -27,3 +27,25 @@ def test_named_barriers_take_diverged_warps():
             used += 1
             assert "__syncwarp();" in src[:m.start()].rsplit("{", 1)[1], fn
     assert used == 2
+
+
+def test_dependent_launches_keep_their_rule():
+    """Kernels launched dependently (launch_after) wait for the kernel before them
+    in every thread, and no kernel parameter that points to memory a kernel of
+    the step writes is declared restrict: a read-only load of it could move
+    above the wait.  Porosity and the fixed temperature are constants."""
+    text = "\n".join(sources().values())
+    kernels = set(re.findall(r"launch_after\(\s*(k_\w+)", text))
+    for m in re.finditer(r"launch_after\(\s*kern\b", text):        # the kernel named just before
+        kernels |= set(re.findall(r"\bk_\w+(?=<)", text[:m.start()].rsplit("auto kern", 1)[1]))
+    assert {"k_split2d", "k_tile2d", "k_march2d", "k_collide3", "k_adj_macro"} <= kernels
+    for k in sorted(kernels):
+        m = re.search(r"__global__[^;{]*?\b%s\((.*?)\)\s*\{" % k, text, re.S)
+        assert m, k
+        assert "after_previous();" in text[m.end():].split("__global__", 1)[0], k
+        for arg in re.findall(r"__restrict__\s+(\w+)", m.group(1)):
+            assert arg in ("phi",), (k, arg)
+    for s in ("StepArgs", "AdjArgs", "ReactArgs"):
+        body = re.search(r"struct %s \{(.*?)\n\};" % s, text, re.S).group(1)
+        for arg in re.findall(r"__restrict__\s+(\w+)", body):
+            assert arg in ("phi", "Tfix"), (s, arg)
