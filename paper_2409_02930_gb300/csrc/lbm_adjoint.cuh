@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(64) k_adj_collide(Params<B> p, InletTables<B> 
   s.template from_moments<EN, true>(p, mo, a.phi[n], EN ? B(0) : a.Tfix[n]);
   Grad<B, 2, M, EN> gr, gb;
   const B* __restrict__ mac = a.mac;
-  gr.compute(p, x, y, z, [&](int k, int nb) { return mac[(size_t)k * N + nb]; });
+  gr.compute(p, x, y, [&](int k, int nb) { return mac[(size_t)k * N + nb]; });
   const B* __restrict__ lam1 = a.lam1 + n;
   auto lam = [&](int l, int i) { return lam1[(size_t)(unsigned)(l * 9 + i) * (unsigned)N]; };
   MomentBar<B, M> mb;

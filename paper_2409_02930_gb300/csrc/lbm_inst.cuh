@@ -80,18 +80,16 @@ struct Launch {
     if constexpr (D == 3) collide_any<false>(p, it, a, nullptr, s);
     else launch_after(k_collide<R, D, M, EN>, grid(p.N), block(p.N), 0, s, p, it, a);
   }
-  // fused step, shared-memory halo ring, tile TX x TY marching SEG planes
-  template <int TX, int TY, int SEG>
+  // fused step, shared-memory ring of macro fields, TX columns marching SEG rows
+  template <int TX, int SEG>
   static int fused_tile(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
     static_assert(D == 2, "fused tiles are a 2-D form");
     if (!rows_fit(p.ny, SEG)) return -1;
-    constexpr size_t smem = fused_smem_bytes<R, D, M, EN, TX, TY>();
-    auto kern = k_fused<R, D, M, EN, TX, TY, SEG>;
+    constexpr size_t smem = fused_smem_bytes<R, M, EN, TX>();
+    auto kern = k_fused<R, M, EN, TX, SEG>;
     static bool done = false;
     if (configure(kern, smem, done)) return -1;
-    dim3 g((p.nx + TX - 1) / TX, D == 3 ? (p.ny + TY - 1) / TY : (p.ny + SEG - 1) / SEG,
-           D == 3 ? (p.nz + SEG - 1) / SEG : 1);
-    kern<<<g, TX * TY, smem, s>>>(p, it, a);
+    kern<<<dim3((p.nx + TX - 1) / TX, (p.ny + SEG - 1) / SEG), TX, smem, s>>>(p, it, a);
     return 0;
   }
   // tiles with the populations in registers
@@ -160,12 +158,13 @@ struct Launch {
   // two-pass form whose node update stages each node's pulled populations in shared memory
   template <int TB>
   static int staged(const Params<R>& p, const InletTables<R>& it, const StepArgs<R>& a, cudaStream_t s) {
-    constexpr size_t smem = sizeof(R) * (size_t)n_pops<R, D, M, EN>() * TB;
+    static_assert(D == 2, "populations are staged in 2-D only");
+    constexpr size_t smem = sizeof(R) * (size_t)n_pops2<M, EN>() * TB;
     if constexpr (smem > kMaxSmem) {
       return -1;
     } else {
-      auto kern = k_collide_staged<R, D, M, EN, TB>;
-      auto kmac = k_macro_staged<R, D, M, EN, TB>;
+      auto kern = k_collide_staged<R, M, EN, TB>;
+      auto kmac = k_macro_staged<R, M, EN, TB>;
       static bool done = false, done_mac = false;
       if (configure(kern, smem, done) || configure(kmac, smem, done_mac)) return -1;
       kmac<<<(p.N + TB - 1) / TB, TB, smem, s>>>(p, it, a);
@@ -181,7 +180,7 @@ struct Launch {
         case 2: return march2d<32, 8, 1, 1>(p, it, a, s);
         case 3: return march2d<128, 4, 1, 1>(p, it, a, s);
         case 4: return march2d<64, 16, 1, 1>(p, it, a, s);
-        case 5: return fused_tile<32, 1, 8>(p, it, a, s);
+        case 5: return fused_tile<32, 8>(p, it, a, s);
         case 6: return staged<64>(p, it, a, s);
         case 7: return staged<128>(p, it, a, s);
         case 8: return march2d_tma<32, 8, 1, 1>(p, it, a, s);

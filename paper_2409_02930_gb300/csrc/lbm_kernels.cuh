@@ -37,14 +37,15 @@ LBM_HD void node_xyz(const Params<R>& p, int n, int& x, int& y, int& z) {
   z = (D == 3) ? r / p.ny : 0;
 }
 
-// Gradient inputs at node (x, y, z) from the neighbours' macro fields
-// (isotropic stencil; zero-gradient copy across non-periodic x faces).
+// Gradient inputs of a node; compute() takes them from the neighbours' macro
+// fields on a D2Q9 lattice (isotropic stencil; zero-gradient copy across
+// non-periodic x faces).  D3Q27 differentiates in lbm_split3d.cuh.
 template <class R, int D, int M, bool EN>
 struct Grad {
   R divu, dPi[D], dY[M][D];
   template <class Fetch>
-  LBM_HD void compute(const Params<R>& p, int x, int y, int z, Fetch&& fetch) {
-    constexpr int Q = Lat<D>::Q;
+  LBM_HD void compute(const Params<R>& p, int x, int y, Fetch&& fetch) {
+    static_assert(D == 2, "the gather stencil is a 2-D form");
     divu = R(0);
 #pragma unroll
     for (int b = 0; b < D; ++b) {
@@ -52,16 +53,14 @@ struct Grad {
 #pragma unroll
       for (int k = 0; k < M; ++k) dY[k][b] = R(0);
     }
-    Unroll<0, Q>::run([&](auto ic) {
+    Unroll<0, 9>::run([&](auto ic) {
       constexpr int I = decltype(ic)::value;
       if (csq_of<D>(I) == 0) return;
       const R w = grad_w<R, D>(I);
       int sx = x + c_of<D>(I, 0);
       if (sx < 0) sx = (p.bc_lo == BC_PERIODIC) ? sx + p.nx : 0;
       if (sx >= p.nx) sx = (p.bc_hi == BC_PERIODIC) ? sx - p.nx : p.nx - 1;
-      int sy = wrapi(y + c_of<D>(I, 1), p.ny);
-      int sz = (D == 3) ? wrapi(z + c_of<D>(I, 2), p.nz) : 0;
-      int nb = sx + p.nx * (sy + p.ny * sz);
+      const int nb = sx + p.nx * wrapi(y + c_of<D>(I, 1), p.ny);
 #pragma unroll
       for (int b = 0; b < D; ++b) {
         const int cb = c_of<D>(I, b);

@@ -61,7 +61,7 @@ LBM_HD void collide_node(const Params<R>& p, const InletTables<R>& it, const Ste
   Grad<R, D, M, EN> gr;
   const R* __restrict__ mac = a.mac;
   const int N = p.N;
-  gr.compute(p, x, y, z, [&](int k, int nb) { return mac[(size_t)k * N + nb]; });
+  gr.compute(p, x, y, [&](int k, int nb) { return mac[(size_t)k * N + nb]; });
   collide_gen<R, D, M, EN>(p, pf, n, mo, s, gr, a.dst, a.status);
 }
 
