@@ -334,8 +334,10 @@ int lbm_get_timing(lbm_ctx* ctx, double* ms_by_kind /* [3] */, long long* launch
  * 3-D and, in 2-D, variant 8 on FP32 lattices with nx a multiple of 4 and no
  * reservoir face of at least 3 * 2^20 nodes, or of at least 2^18 in at most 1216
  * blocks of 30 x 8 nodes, else tiles (10 up to 9728 nodes, above
- * that 12 in FP32 and 11 in FP64; lattices of one or two rows with 8192 nodes
- * or more: the two-pass form); batches use variant 10.  The adjoint's
+ * that 12 in FP32 and 11 in FP64).  The two-pass form serves lattices of one or
+ * two rows with 8192 nodes or more, and lattices narrower than a tile once
+ * their tiles are more than a few per SM (fewer than 20 columns in FP32 or 32
+ * in FP64, fewer than 8 up to 9728 nodes).  Batches use variant 10.  The adjoint's
  * forward and recompute steps use the context's form.  lbm_autotune times
  * every form for `steps` steps on the
  * current state, restores the state, selects the fastest form and writes its

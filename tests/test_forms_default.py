@@ -53,12 +53,42 @@ def test_default_form_at_its_lines(rule):
         assert form(rule, 64, 153, fp64=fp64) == tile
         assert form(rule, 4095, 2, fp64=fp64) == 10
         assert form(rule, 4096, 2, fp64=fp64) == -1
-        assert form(rule, 4, 4 * 65535, fp64=fp64) == tile
-        assert form(rule, 4, 4 * 65535 + 1, fp64=fp64) == -1
+        assert form(rule, 32, 4 * 65535, fp64=fp64, bc=1) == tile
+        assert form(rule, 32, 4 * 65535 + 1, fp64=fp64, bc=1) == -1
         assert form(rule, 2048, 1535, fp64=fp64) == tile
         assert form(rule, 2048, 1536, fp64=fp64) == (8 if not fp64 else tile)
         assert form(rule, 2048, 1536, fp64=fp64, bc=1) == tile
         assert form(rule, 2050, 1536, fp64=fp64) == tile
-    assert form(rule, 8, 8 * 65535) == 8
-    assert form(rule, 8, 8 * 65535 + 1) == -1
+    assert form(rule, 20, 8 * 65535) == 8
+    assert form(rule, 20, 8 * 65535 + 1) == -1
     assert form(rule, 12, 4, nz=4) == 5
+
+
+@pytest.mark.parametrize("bc", [0, 1, 2])
+def test_narrow_lattices_leave_the_tiles(rule, bc):
+    """Lattices narrower than a tile run in two passes once their tiles are more
+    than a few per SM, and on tiles on the other side of each line."""
+    for fp64 in (False, True):
+        for nx, ny in ((1, 200000), (2, 100003), (3, 66669), (4, 50003), (6, 33336), (8, 25003), (1, 9000), (1, 10000),
+                       (3, 20000), (2, 5000), (4, 2500)):
+            assert form(rule, nx, ny, fp64=fp64, bc=bc) == -1, (nx, ny, fp64)
+    # FP32: 8 x 4 tiles up to four per SM, 32 x 4 tiles up to three, 20 columns
+    assert form(rule, 1, 4 * 608, bc=bc) == 10
+    assert form(rule, 1, 4 * 608 + 1, bc=bc) == -1
+    assert form(rule, 7, 1389, bc=bc) == 10
+    assert form(rule, 16, 4 * 456, bc=bc) == 12
+    assert form(rule, 16, 4 * 456 + 1, bc=bc) == -1
+    assert form(rule, 19, 11000, bc=bc) == -1
+    assert form(rule, 20, 11000, bc=bc) == 12
+    # FP64: 8 x 4 tiles up to three per SM, 16 x 8 tiles by waves
+    assert form(rule, 1, 4 * 456, fp64=True, bc=bc) == 10
+    assert form(rule, 1, 4 * 456 + 1, fp64=True, bc=bc) == -1
+    assert form(rule, 8, 1250, fp64=True, bc=bc) == -1
+    assert form(rule, 12, 2000, fp64=True, bc=bc) == 11
+    assert form(rule, 12, 16669, fp64=True, bc=bc) == -1
+    assert form(rule, 14, 14288, fp64=True, bc=bc) == 11
+    assert form(rule, 16, 12503, fp64=True, bc=bc) == 11
+    assert form(rule, 17, 11767, fp64=True, bc=bc) == -1
+    assert form(rule, 24, 1000, fp64=True, bc=bc) == 11
+    assert form(rule, 31, 6454, fp64=True, bc=bc) == 11
+    assert form(rule, 32, 6253, fp64=True, bc=bc) == 11
