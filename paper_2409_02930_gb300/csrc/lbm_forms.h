@@ -15,20 +15,21 @@ inline bool rows_fit(long long ny, int rows) { return (ny + rows - 1) / rows <= 
 // every block still pays for the whole tile, so beyond a few blocks per SM they
 // take the two-pass form, whose threads all have a node.  us per step (tiles /
 // two-pass), FP32 in tiles of 32 x 4: 1x200000 579 / 32, 8x25003 77 / 33,
-// 18x11114 36.8 / 34.2, 20x10003 33.2 / 34.2; 12x2000 (500 tiles) 10.7 / 7.2,
-// 16x1500 (375) 6.4 / 7.1.  FP64 in tiles of 16 x 8: 1x200000 6192 / 525,
+// 18x11114 36.8 / 34.2, 20x10003 33.2 / 34.2; 12x2500 (625 tiles) 10.9 / 7.3
+// (two isothermal species 11.1 / 7.4, and 7.1 / 7.8 at 19x1900, 475).  FP64 in tiles of 16 x 8: 1x200000 6192 / 525,
 // 10x20003 646 / 527, 12x16669 533 / 527, 14x14288 459 / 526, 16x12503 420 / 525,
 // 17x11767 757 / 528, 24x8336 534 / 526, 28x7145 459 / 527 (isothermal 18x8000
 // 418 / 267): about 39 us for every 152 tiles against 45 us for every 152 x 128
-// nodes in two passes (8x1250 78 / 47, 12x2000 78 / 90, 24x1000 78 / 90).  Split by lattice, tiles of 8 x 4: FP32 1x2000 (500
-// tiles) 6.2 / 5.7, 4x2400 (600) 6.6 / 6.6, 3x3200 (800) 7.6 / 6.7, 1x9000 16.7 /
-// 6.3; FP64 6x1600 (400) 43.9 / 44.8, 5x1900 (475) 50.7 / 45.1, 1x9000 197 / 45.
+// nodes in two passes (8x1250 78 / 47, 24x800 78 / 48, 12x2000 78 / 90, 24x1000 78 / 90).  Split by
+// lattice, tiles of 8 x 4: FP32 4x2400 (600 tiles) 6.6 / 6.6, 1x9000 (2,250) 16.7 /
+// 6.3 (two isothermal species 11.1 / 7.4, and 4.0 / 7.1 with 475); FP64 6x1600 (400)
+// 43.9 / 44.8, 5x1900 (475) 50.7 / 45.1, 1x9000 197 / 45.
 constexpr int kSMs = 152;
 constexpr long long kSplit2dNodes = 2 * kSMs * 32, kMarchNodes = 3 << 20;
 inline bool narrow_lattice(long long nx, long long ny, bool single) {
   auto rows = [&](int t) { return (ny + t - 1) / t; };
-  if (nx * ny <= kSplit2dNodes) return nx < 8 && rows(4) > (single ? 4 : 3) * kSMs;
-  if (single) return nx < 20 && rows(4) > 3 * kSMs;
+  if (nx * ny <= kSplit2dNodes) return nx < 8 && rows(4) > (single ? 8 : 3) * kSMs;
+  if (single) return nx < 20 && rows(4) > 4 * kSMs;
   const long long tiles = (nx + 15) / 16 * rows(8);
   return nx < 32 && 5 * ((tiles + kSMs - 1) / kSMs) > 6 * ((nx * ny + kSMs * 128 - 1) / (kSMs * 128));
 }

@@ -23,7 +23,7 @@ def rule(tmp_path_factory):
                    % os.path.join(ROOT, "paper_2409_02930_gb300", "csrc", "lbm_forms.h"))
     so = d / "forms.so"
     subprocess.run([cxx, "-std=c++17", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
-    return ctypes.CDLL(str(so)).form
+    return ctypes.CDLL(str(so))
 
 
 def form(rule, nx, ny, nz=1, fp64=False, bc=0):
@@ -31,7 +31,7 @@ def form(rule, nx, ny, nz=1, fp64=False, bc=0):
     c = lbm.LbmConfig()
     c.nx, c.ny, c.nz, c.bc_lo, c.bc_hi = nx, ny, nz, bc, bc
     c.precision = lbm.LBM_FP64 if fp64 else lbm.LBM_FP32
-    return rule(ctypes.byref(c))
+    return rule.form(ctypes.byref(c))
 
 
 @pytest.mark.parametrize("fp64", [False, True])
@@ -72,12 +72,12 @@ def test_narrow_lattices_leave_the_tiles(rule, bc):
         for nx, ny in ((1, 200000), (2, 100003), (3, 66669), (4, 50003), (6, 33336), (8, 25003), (1, 9000), (1, 10000),
                        (3, 20000), (2, 5000), (4, 2500)):
             assert form(rule, nx, ny, fp64=fp64, bc=bc) == -1, (nx, ny, fp64)
-    # FP32: 8 x 4 tiles up to four per SM, 32 x 4 tiles up to three, 20 columns
-    assert form(rule, 1, 4 * 608, bc=bc) == 10
-    assert form(rule, 1, 4 * 608 + 1, bc=bc) == -1
+    # FP32: 8 x 4 tiles up to eight per SM, 32 x 4 tiles up to four, 20 columns
+    assert form(rule, 1, 4 * 1216, bc=bc) == 10
+    assert form(rule, 1, 4 * 1216 + 1, bc=bc) == -1
     assert form(rule, 7, 1389, bc=bc) == 10
-    assert form(rule, 16, 4 * 456, bc=bc) == 12
-    assert form(rule, 16, 4 * 456 + 1, bc=bc) == -1
+    assert form(rule, 16, 4 * 608, bc=bc) == 12
+    assert form(rule, 16, 4 * 608 + 1, bc=bc) == -1
     assert form(rule, 19, 11000, bc=bc) == -1
     assert form(rule, 20, 11000, bc=bc) == 12
     # FP64: 8 x 4 tiles up to three per SM, 16 x 8 tiles by waves
