@@ -337,7 +337,9 @@ int lbm_get_timing(lbm_ctx* ctx, double* ms_by_kind /* [3] */, long long* launch
  * that 12 in FP32 and 11 in FP64).  The two-pass form serves lattices of one or
  * two rows with 8192 nodes or more, and lattices narrower than a tile once
  * their tiles are more than a few per SM (fewer than 20 columns in FP32 or 32
- * in FP64, fewer than 8 up to 9728 nodes).  Batches use variant 10.  The adjoint's
+ * in FP64, fewer than 8 up to 9728 nodes).  Batches use variant 10, or variant 0 where
+ * their tiles are many and two fifths (FP64: a tenth) of the tiles' nodes lie
+ * outside the lattices.  The adjoint's
  * forward and recompute steps use the context's form.  lbm_autotune times
  * every form for `steps` steps on the
  * current state, restores the state, selects the fastest form and writes its

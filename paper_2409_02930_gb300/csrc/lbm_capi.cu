@@ -499,7 +499,7 @@ int lbm_create_batch(lbm_ctx** out, int n_cases, const lbm_config* cfgs) {
   x->precision = c0.precision;
   x->stream = (cudaStream_t)c0.stream;
   x->n_cases = n_cases;
-  x->variant = 10;                      // one pass over 32 x 4 tiles, resident blocks looping over them
+  x->variant = lbm::default_batch_variant(n_cases, cfgs);
   bool ok = (x->precision == LBM_FP64)
                 ? lbm::get_ops_f64_2d(x->M, x->energy, &x->od) && lbm::get_batch_ops_f64(x->M, x->energy, &x->bd)
                 : lbm::get_ops_f32_2d(x->M, x->energy, &x->of) && lbm::get_batch_ops_f32(x->M, x->energy, &x->bf);

@@ -1,5 +1,5 @@
-// Which kernel form a new single lattice takes, from its configuration alone
-// (host code without CUDA).
+// Which kernel form a new single lattice or batch takes, from its configuration
+// alone (host code without CUDA).
 #pragma once
 
 #include "../../include/lbm.h"
@@ -62,6 +62,28 @@ inline int default_variant(const lbm_config* c) {
   if (single && !reservoir && (one_wave || N >= kMarchNodes) && c->nx % 4 == 0 && rows_fit(c->ny, 8)) return 8;
   if (!rows_fit(c->ny, 4) || (c->ny < 3 && N >= 8192)) return -1;
   return N <= kSplit2dNodes ? 10 : (single ? 12 : 11);
+}
+
+// Kernel form of a new batch: tiles of 32 x 4 nodes (10), or two passes over runs
+// of 64 nodes (0) where the cases are so narrow or of so few rows that too many
+// of the tiles' threads have no node, and the tiles are more than the SMs hold
+// at once.  us per step (tiles / runs), cases x their sizes, energy lattice with
+// three species unless said: FP32 8 x 3x5000 119 / 19, 8 x 12x2000 50 / 27, 8 x
+// 22x600 18.8 / 15.2 but two isothermal species 13.7 / 15.8, 8 x 28x600 19.1 / 20.3,
+// 64 tubes of one row 15.9 / 9.8, of two 16.8 / 15.9, of three 18.7 / 21.6; FP64
+// 8 x 3x5000 2592 / 315, 8 x 22x600 317 / 238, 8 x 28x600 318 / 317 (two species 274 /
+// 244), 8 x 30x600 319 / 317 (273 / 283), tubes of three rows 326 / 306, of four 403 /
+// 413.  By tiles: FP32 two species 16 x 12x100 (400 tiles) 7.0 / 7.6, 24 x 12x100
+// (600) 7.6 / 8.0; FP64 8 x 5x200 (400) 161 / 42, 8 tubes of nine rows (130) 38 / 37.
+inline int default_batch_variant(int n_cases, const lbm_config* cfgs) {
+  long long nodes = 0, tiles = 0;
+  for (int c = 0; c < n_cases; ++c) {
+    nodes += (long long)cfgs[c].nx * cfgs[c].ny;
+    tiles += ((cfgs[c].nx + 31LL) / 32) * ((cfgs[c].ny + 3LL) / 4);
+  }
+  const bool single = cfgs[0].precision == LBM_FP32;
+  const bool idle = 10 * nodes < (single ? 6 : 9) * 128 * tiles;
+  return idle && tiles > (single ? 4 : 1) * kSMs ? 0 : 10;
 }
 
 }  // namespace lbm

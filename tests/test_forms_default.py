@@ -20,6 +20,7 @@ def rule(tmp_path_factory):
     d = tmp_path_factory.mktemp("forms")
     src = d / "forms.cpp"
     src.write_text('#include "%s"\nextern "C" int form(const lbm_config* c) { return lbm::default_variant(c); }\n'
+                   'extern "C" int batch_form(int n, const lbm_config* c) { return lbm::default_batch_variant(n, c); }\n'
                    % os.path.join(ROOT, "paper_2409_02930_gb300", "csrc", "lbm_forms.h"))
     so = d / "forms.so"
     subprocess.run([cxx, "-std=c++17", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
@@ -92,3 +93,31 @@ def test_narrow_lattices_leave_the_tiles(rule, bc):
     assert form(rule, 24, 1000, fp64=True, bc=bc) == 11
     assert form(rule, 31, 6454, fp64=True, bc=bc) == 11
     assert form(rule, 32, 6253, fp64=True, bc=bc) == 11
+
+
+def batch_form(rule, cases, fp64=False):
+    from paper_2409_02930_gb300 import lbm
+    cs = (lbm.LbmConfig * len(cases))()
+    for c, (nx, ny) in zip(cs, cases):
+        c.nx, c.ny, c.nz = nx, ny, 1
+        c.precision = lbm.LBM_FP64 if fp64 else lbm.LBM_FP32
+    return rule.batch_form(len(cases), cs)
+
+
+def test_batches_of_narrow_cases_leave_the_tiles(rule):
+    for fp64 in (False, True):
+        for nx, ny, n in ((3, 5000, 8), (4, 2000, 8), (8, 3000, 8), (12, 2000, 8), (19, 2000, 8), (3, 40000, 2)):
+            assert batch_form(rule, [(nx, ny)] * n, fp64) == 0, (nx, ny, fp64)
+        assert batch_form(rule, [(1000, 4)] * 64, fp64) == 10
+        assert batch_form(rule, [(1000, 1)] * 64, fp64) == 0
+        assert batch_form(rule, [(20, 30)], fp64) == 10
+        assert batch_form(rule, [(1000, 2)] * 64, fp64) == 0
+        assert batch_form(rule, [(1000, 3)] * 64, fp64) == (0 if fp64 else 10)
+    assert batch_form(rule, [(20, 2000)] * 8) == 10                  # three fifths of each tile
+    assert batch_form(rule, [(5, 200)] * 12) == 10                   # 600 tiles
+    assert batch_form(rule, [(5, 200)] * 13) == 0
+    assert batch_form(rule, [(24, 2000)] * 8, fp64=True) == 0
+    assert batch_form(rule, [(29, 2000)] * 8, fp64=True) == 10       # nine tenths
+    assert batch_form(rule, [(5, 200)] * 3, fp64=True) == 10         # 150 tiles
+    assert batch_form(rule, [(5, 200)] * 8, fp64=True) == 0
+    assert batch_form(rule, [(5, 200)] * 8 + [(2048, 256)], fp64=True) == 10
