@@ -325,10 +325,14 @@ int lbm_get_timing(lbm_ctx* ctx, double* ms_by_kind /* [3] */, long long* launch
  * the same tile shape, variants 2 and 0), 10 the single-launch form on tiles
  * of 8 x 4 nodes with one warp per lattice, 11-12 the single-launch form on
  * tiles of 16 x 8 and 32 x 4 nodes with a node's populations in one thread.
- * D3Q27: every form is the two-pass step split by lattice (one warp per
- * lattice of 32 nodes); the indices select the registers a thread may use
- * (0: one resident block per SM, 1: two, 2: three, 3: four; 4 and 5 the
- * default).  Every form
+ * D3Q27: every form is the two-pass step split by lattice.  Indices 3, 4, 5
+ * and -1 are one form, the default: blocks of 32 nodes with one warp per
+ * lattice, registers for two resident blocks per SM; in FP32 the populations
+ * wait in shared memory between their sums and their relaxation, in FP64
+ * lattices up to 608 nodes run in blocks of 8 nodes and up to 4864 in blocks of
+ * 16.  Indices 0, 1 and 2 always take 32 nodes and keep the populations in
+ * registers, as many as leave one, two or three resident blocks per SM (FP64: 2
+ * as 1).  Every form
  * computes the same step (the gradient stencil is summed in different
  * orders, so the forms agree to rounding).  New contexts use variant 5 in
  * 3-D and, in 2-D, variant 8 on FP32 lattices with nx a multiple of 4 and no
@@ -341,7 +345,7 @@ int lbm_get_timing(lbm_ctx* ctx, double* ms_by_kind /* [3] */, long long* launch
  * their tiles are many and two fifths (FP64: a tenth) of the tiles' nodes lie
  * outside the lattices.  The adjoint's
  * forward and recompute steps use the context's form.  lbm_autotune times
- * every form for `steps` steps on the
+ * every form (of indices that are one form the highest) for `steps` steps on the
  * current state, restores the state, selects the fastest form and writes its
  * index to *best (may be NULL).  Errors: LBM_ERR_ARG (unknown variant,
  * steps < 1), LBM_ERR_ALLOC.

@@ -907,6 +907,7 @@ int lbm_autotune(lbm_ctx* x, int steps, int* best) {
   int best_v = var0;
   const int nv = lbm_variant_count(x);
   for (int v = (x->n_cases > 0 ? 0 : -1); v < nv && e == cudaSuccess; ++v) {
+    if (lbm::alias_form(x->D, x->precision == LBM_FP32, v)) continue;
     x->variant = v;
     if (step_once(x) != LBM_OK) continue;           // warm-up (also configures the kernel)
     cudaEventRecord(t0, x->stream);

@@ -64,6 +64,13 @@ inline int default_variant(const lbm_config* c) {
   return N <= kSplit2dNodes ? 10 : (single ? 12 : 11);
 }
 
+// Form indices that launch the same kernels as another one, so that a search
+// over the forms times each once: of the D3Q27 indices 3, 4 and -1 are the
+// default form 5, and in FP64 2 is 1.
+inline bool alias_form(int D, bool single, int v) {
+  return D == 3 && (v == -1 || v == 3 || v == 4 || (v == 2 && !single));
+}
+
 // Kernel form of a new batch: tiles of 32 x 4 nodes (10), or two passes over runs
 // of 64 nodes (0) where the cases are so narrow or of so few rows that too many
 // of the tiles' threads have no node, and the tiles are more than the SMs hold

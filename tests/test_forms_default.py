@@ -21,6 +21,7 @@ def rule(tmp_path_factory):
     src = d / "forms.cpp"
     src.write_text('#include "%s"\nextern "C" int form(const lbm_config* c) { return lbm::default_variant(c); }\n'
                    'extern "C" int batch_form(int n, const lbm_config* c) { return lbm::default_batch_variant(n, c); }\n'
+                   'extern "C" int alias(int D, int single, int v) { return lbm::alias_form(D, single != 0, v); }\n'
                    % os.path.join(ROOT, "paper_2409_02930_gb300", "csrc", "lbm_forms.h"))
     so = d / "forms.so"
     subprocess.run([cxx, "-std=c++17", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
@@ -121,3 +122,10 @@ def test_batches_of_narrow_cases_leave_the_tiles(rule):
     assert batch_form(rule, [(5, 200)] * 3, fp64=True) == 10         # 150 tiles
     assert batch_form(rule, [(5, 200)] * 8, fp64=True) == 0
     assert batch_form(rule, [(5, 200)] * 8 + [(2048, 256)], fp64=True) == 10
+
+
+def test_alias_indices(rule):
+    """Indices that a search over the forms passes over; each is one of the others."""
+    for single in (0, 1):
+        assert not any(rule.alias(2, single, v) for v in range(-1, 13))
+        assert [v for v in range(-1, 6) if not rule.alias(3, single, v)] == ([0, 1, 2, 5] if single else [0, 1, 5])

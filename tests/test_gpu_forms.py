@@ -217,3 +217,24 @@ def test_surface_source_of_low_rank_mechanisms(L, steps):
         assert worst(g.populations(), o.pops()) < 1e-12
         assert np.max(np.abs(g.moments(L.LBM_MOM_XS) - o.moments(oracle.MOM_XS))) < 1e-12
         g.close()
+
+
+@pytest.mark.parametrize("shape", [(7, 4, 3), (33, 9, 5), (21, 18, 16)])
+def test_indices_that_are_one_form(L, shape):
+    """D3Q27 indices that name one form return the same bits, and the autotuner
+    settles on one of the forms that differ."""
+    wl = anode(*shape)
+    for prec in (L.LBM_FP64, L.LBM_FP32):
+        pops = {}
+        for v in (-1, 0, 1, 2, 3, 4, 5):
+            g = L.Lattice(wl, precision=prec)
+            g.set_variant(v)
+            g.step(2)
+            g.sync()
+            pops[v] = g.populations()
+            g.close()
+        same = [(-1, 5), (3, 5), (4, 5)] + ([(1, 2)] if prec == L.LBM_FP64 else [])
+        assert all(np.array_equal(pops[a], pops[b]) for a, b in same)
+        g = L.Lattice(wl, precision=prec)
+        assert g.autotune(2) in ((0, 1, 2, 5) if prec == L.LBM_FP32 else (0, 1, 5))
+        g.close()
