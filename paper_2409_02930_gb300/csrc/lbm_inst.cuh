@@ -218,7 +218,7 @@ struct Launch {
     if constexpr (has_react) {
       R* aux = a.mac + (size_t)(2 * D + M) * p.N;
       macro_any<true>(p, it, a, aux, s);
-      if (p.N <= source_warp_nodes) {
+      if (p.N <= source_warp_nodes<R>) {
         launch_after(k_source_warp<R, M>, p.N, 32, 0, s, p.N, aux, a.phi, a.status, ra);
       } else if (p.N <= source_wide_nodes) {
         k_source<R, M, 1><<<(p.N + 127) / 128, 128, 0, s>>>(p.N, aux, a.phi, a.status, ra);

@@ -349,15 +349,17 @@ __global__ void __launch_bounds__(128, MINB) k_source(int N, const R* aux, const
   for (int k = 0; k < mc.S; ++k) ra.Xs_out[(size_t)k * N + n] = Xs1[k];
 }
 
-// Which form a lattice of N nodes takes.  A warp per node up to 2048 nodes
-// (measured before the solve in r changes, FP64 12 x 2 x 2: 157 us per reactive
-// step against 380 us with a thread per node; 8192 nodes FP32 376 against 303, so the line lies below 152 SMs x a few
-// warps).  Above it a thread per node: without a register limit while the
-// threads do not fill the GPU (8192 nodes FP32 303 us per step at 222
-// registers, 332 at 48), then limited to 48 (FP32) or 64 (FP64) registers, so
-// that more threads hide the latency of the work arrays (524,288 nodes FP32
-// 5.58 -> 4.45 ms per step).
-constexpr int source_warp_nodes = 2048;
+// Which form a lattice of N nodes takes; us per reactive step of a D3Q27 anode.
+// A warp per node up to 48 (FP32) or 32 (FP64) nodes per SM: its time grows with
+// the nodes, a thread per node takes one node's latency until the threads fill
+// the GPU (warp / thread: FP32 2,048 nodes 126 / 278, 4,096 181 / 283, 7,168 241 /
+// 287, 7,680 281 / 289, 8,192 287 / 287; FP64 48 nodes 101 / 294, 2,048 197 / 367,
+// 4,864 350 / 413, 6,144 493 / 442).  Above it a thread per node: without a
+// register limit up to two blocks of 128 threads per SM, then limited to 48 (FP32)
+// or 64 (FP64) registers, so that more threads hide the latency of the work arrays
+// (none / limited: FP32 16,384 nodes 303 / 326, 38,912 431 / 481, 65,536 763 / 648;
+// FP64 616 / 642, 1,010 / 1,055, 1,663 / 1,530).
+template <class R> constexpr int source_warp_nodes = 152 * (sizeof(R) == 4 ? 48 : 32);
 constexpr int source_wide_nodes = 152 * 128 * 2;
 
 // The same source with one warp per node, for lattices too small to fill the

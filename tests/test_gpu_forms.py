@@ -238,3 +238,42 @@ def test_indices_that_are_one_form(L, shape):
         g = L.Lattice(wl, precision=prec)
         assert g.autotune(2) in ((0, 1, 2, 5) if prec == L.LBM_FP32 else (0, 1, 5))
         g.close()
+
+
+# a warp per node up to 7,296 (FP32) and 4,864 (FP64) nodes, one past the line,
+# and inside the thread form without a register limit
+@pytest.mark.parametrize("shape,precision", [((19, 16, 16), "fp64"), ((17, 41, 7), "fp64"), ((32, 16, 12), "fp64"),
+                                             ((19, 24, 16), "fp32"), ((8, 48, 20), "fp32"), ((24, 20, 18), "fp32")])
+def test_surface_source_at_its_lines(L, shape, precision):
+    """FP64 within the parity bound; in FP32 the populations within 16 roundings a
+    step and the coverages, which are FP64, within 1e-8, the bound of the tests at
+    full size."""
+    wl = W.anode3d_reactive(*shape, steps=2)
+    o = oracle.Oracle(wl)
+    o.step(2)
+    fp64 = precision == "fp64"
+    g = L.Lattice(wl, precision=L.LBM_FP64 if fp64 else L.LBM_FP32)
+    g.step(2)
+    g.sync()
+    assert worst(g.populations(), o.pops()) < (1e-12 if fp64 else 16 * 2 * 2.0 ** -24)
+    assert np.max(np.abs(g.moments(L.LBM_MOM_XS) - o.moments(oracle.MOM_XS))) < (1e-12 if fp64 else 1e-8)
+    g.close()
+
+
+@pytest.mark.parametrize("steps", [1, 7])
+def test_thread_form_of_low_rank_mechanisms(L, steps):
+    """As test_surface_source_of_low_rank_mechanisms, on a lattice above the warp
+    form's line."""
+    mc = W.surface_mechanism()
+    for k in ("nu_gas", "nu_surf", "A", "Ea"):
+        setattr(mc, k, np.ascontiguousarray(getattr(mc, k)[:steps]))
+    mc.R = steps
+    wl = W.anode3d(17, 41, 7, mechanism=mc, steps=2)
+    o = oracle.Oracle(wl)
+    o.step(2)
+    g = L.Lattice(wl, precision=L.LBM_FP64)
+    g.step(2)
+    g.sync()
+    assert worst(g.populations(), o.pops()) < 1e-12
+    assert np.max(np.abs(g.moments(L.LBM_MOM_XS) - o.moments(oracle.MOM_XS))) < 1e-12
+    g.close()
