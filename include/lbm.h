@@ -346,8 +346,9 @@ int lbm_get_timing(lbm_ctx* ctx, double* ms_by_kind /* [3] */, long long* launch
  * outside the lattices.  The adjoint's
  * forward and recompute steps use the context's form.  lbm_autotune times
  * every form (of indices that are one form the highest) for `steps` steps on the
- * current state, restores the state, selects the fastest form and writes its
- * index to *best (may be NULL).  Errors: LBM_ERR_ARG (unknown variant,
+ * current state, restores the state, selects the fastest form (the one in effect
+ * unless another takes less than 98 % of its time) and writes its index to *best
+ * (may be NULL).  Errors: LBM_ERR_ARG (unknown variant,
  * steps < 1), LBM_ERR_ALLOC.
  */
 int lbm_variant_count(const lbm_ctx* ctx);

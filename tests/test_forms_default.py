@@ -22,6 +22,7 @@ def rule(tmp_path_factory):
     src.write_text('#include "%s"\nextern "C" int form(const lbm_config* c) { return lbm::default_variant(c); }\n'
                    'extern "C" int batch_form(int n, const lbm_config* c) { return lbm::default_batch_variant(n, c); }\n'
                    'extern "C" int alias(int D, int single, int v) { return lbm::alias_form(D, single != 0, v); }\n'
+                   'extern "C" int settled(int h, float hm, int b, float bm) { return lbm::settled_form(h, hm, b, bm); }\n'
                    % os.path.join(ROOT, "paper_2409_02930_gb300", "csrc", "lbm_forms.h"))
     so = d / "forms.so"
     subprocess.run([cxx, "-std=c++17", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
@@ -129,3 +130,11 @@ def test_alias_indices(rule):
     for single in (0, 1):
         assert not any(rule.alias(2, single, v) for v in range(-1, 13))
         assert [v for v in range(-1, 6) if not rule.alias(3, single, v)] == ([0, 1, 2, 5] if single else [0, 1, 5])
+
+
+def test_search_keeps_the_form_in_effect_on_near_ties(rule):
+    rule.settled.argtypes = [ctypes.c_int, ctypes.c_float, ctypes.c_int, ctypes.c_float]
+    assert rule.settled(8, 27.5, 12, 27.4) == 8
+    assert rule.settled(8, 27.5, 12, 26.9) == 12
+    assert rule.settled(8, 27.5, 8, 27.5) == 8
+    assert rule.settled(3, 0.0, 5, 27.5) == 5                # the form in effect was not timed
