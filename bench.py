@@ -575,25 +575,37 @@ def run_reference(args, ws, rank):
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
 
 
-PROFILE_FORMS = ("slab", "slab_fp64", "slab2048", "anode", "anode_gather", "react", "batch", "adjoint")
+PROFILE_FORMS = ("slab", "slab_fp64", "slab2048", "slab_small", "capillary", "anode", "anode_gather", "react", "halfcell",
+                 "batch", "adjoint")
 
 
 def profile_form(which):
     """A few steps of one kernel form on a small case, for a profiler run
     (ncu); prints nothing but "ok".
     slab: the 512x512 slab in FP32, default form (TMA row march), 3 steps;
-    slab_fp64: the same in FP64;
+    slab_fp64: the same in FP64 (tiles of 16 x 8 nodes);
     slab2048: the 2048x2048 slab in FP32 (the back-to-back line), 3 steps;
+    slab_small: the 64x40 slab in FP32, capillary: the 256x4 tube in FP64 (one
+      warp per lattice, variant 10), 3 steps;
     anode: D3Q27 anode 64x32x32, six species, FP32, the default form (split by
-      lattice, variant 5), 3 steps; anode_gather: the same step as variant 3;
+      lattice, variant 5), 3 steps; anode_gather: the same under its index 3;
     react: the same lattice with the seeded surface mechanism, FP32, 3 steps;
-    batch: the 64-capillary sweep, FP32, one block per 8 x 4 tile (variant 7),
-      5 steps launched one by one (timing on, so no graph replay);
+    halfcell: the 12x2x2 electrochemical anode in FP64, 3 steps;
+    batch: the 64-capillary sweep, FP32, its default form (tiles of 32 x 4 nodes,
+      variant 10), 5 steps launched one by one (timing on, so no graph replay);
     adjoint: 64x64 adjoint slab, FP32, 10 steps with checkpoints every 5."""
     from paper_2409_02930_gb300 import lbm
     if which in ("slab", "slab_fp64", "slab2048"):
         side = 2048 if which == "slab2048" else 512
         g = lbm.Lattice(W.slab(side, side, steps=3), precision=lbm.LBM_FP64 if which == "slab_fp64" else lbm.LBM_FP32)
+        g.step(3)
+        g.sync()
+    elif which == "slab_small":
+        g = lbm.Lattice(W.slab(64, 40, steps=3), precision=lbm.LBM_FP32)
+        g.step(3)
+        g.sync()
+    elif which == "capillary":
+        g = lbm.Lattice(W.capillary(256, 4, steps=3), precision=lbm.LBM_FP64)
         g.step(3)
         g.sync()
     elif which in ("anode", "anode_gather"):
@@ -605,9 +617,12 @@ def profile_form(which):
         g = lbm.Lattice(W.anode3d_reactive(nx=64, ny=32, nz=32, steps=3), precision=lbm.LBM_FP32)
         g.step(3)
         g.sync()
+    elif which == "halfcell":
+        g = lbm.Lattice(W.anode3d_electro(nx=12, ny=2, nz=2, steps=3), precision=lbm.LBM_FP64)
+        g.step(3)
+        g.sync()
     elif which == "batch":
         b = lbm.Batch(W.capillary_batch(), precision=lbm.LBM_FP32)
-        b.set_variant(7)
         lbm.load().lbm_set_timing(b._h, 1)
         b.step(5)
         b.sync()

@@ -16,14 +16,15 @@ inline bool rows_fit(long long ny, int rows) { return (ny + rows - 1) / rows <= 
 // take the two-pass form, whose threads all have a node.  us per step (tiles /
 // two-pass), FP32 in tiles of 32 x 4: 1x200000 579 / 32, 8x25003 77 / 33,
 // 18x11114 36.8 / 34.2, 20x10003 33.2 / 34.2; 12x2500 (625 tiles) 10.9 / 7.3
-// (two isothermal species 11.1 / 7.4, and 7.1 / 7.8 at 19x1900, 475).  FP64 in tiles of 16 x 8: 1x200000 6192 / 525,
-// 10x20003 646 / 527, 12x16669 533 / 527, 14x14288 459 / 526, 16x12503 420 / 525,
-// 17x11767 757 / 528, 24x8336 534 / 526, 28x7145 459 / 527 (isothermal 18x8000
-// 418 / 267): about 39 us for every 152 tiles against 45 us for every 152 x 128
-// nodes in two passes (8x1250 78 / 47, 24x800 78 / 48, 12x2000 78 / 90, 24x1000 78 / 90).  Split by
-// lattice, tiles of 8 x 4: FP32 4x2400 (600 tiles) 6.6 / 6.6, 1x9000 (2,250) 16.7 /
-// 6.3 (two isothermal species 11.1 / 7.4, and 4.0 / 7.1 with 475); FP64 6x1600 (400)
-// 43.9 / 44.8, 5x1900 (475) 50.7 / 45.1, 1x9000 197 / 45.
+// (two isothermal species 11.1 / 7.4, and 7.1 / 7.8 at 19x1900, 475 tiles).  FP64
+// in tiles of 16 x 8: 1x200000 6192 / 525, 10x20003 646 / 527, 12x16669 533 / 527,
+// 14x14288 459 / 526, 16x12503 420 / 525, 17x11767 757 / 528, 24x8336 534 / 526,
+// 28x7145 459 / 527 (isothermal 18x8000 418 / 267): about 39 us for every 152 tiles
+// against 45 us for every 152 x 128 nodes in two passes (8x1250 78 / 47, 24x800 78 /
+// 48, 12x2000 78 / 90, 24x1000 78 / 90).  Split by lattice, tiles of 8 x 4: FP32
+// 4x2400 (600 tiles) 6.6 / 6.6, 1x5000 (1,250) 10.3 / 5.7, 1x9000 16.7 / 6.3 (two
+// isothermal species 3x3000, 750 tiles, 5.3 / 6.9, 1x9000 11.1 / 7.4); FP64 6x1600
+// (400) 43.9 / 44.8, 5x1900 (475) 50.7 / 45.1, 1x9000 197 / 45.
 constexpr int kSMs = 152;
 constexpr long long kSplit2dNodes = 2 * kSMs * 32, kMarchNodes = 3 << 20;
 inline bool narrow_lattice(long long nx, long long ny, bool single) {
@@ -36,19 +37,25 @@ inline bool narrow_lattice(long long nx, long long ny, bool single) {
 
 // Kernel form of a new single lattice.  3-D: the split step.  2-D, measured in
 // us per step (tiles / row march): FP32 256x256 with reservoirs 14.4 / 73,
-//   512x512 28.0 / 28.0, 640x512 36.1 / 52.5, 512x768 43.0 / 54.5, 1024x512
+//   512x512 27.5 / 27.4, 640x512 36.1 / 52.5, 512x768 43.0 / 54.5, 1024x512
 //   55.3 / 56.5, 1024x1024 104.6 / 108.4, 1536x1536 224 / 226, 2048x2048 389 /
 //   380, 701x523 with walls 45 / 58; FP64 512x512 549 / 689.
 // The row march (bulk tensor copies, rows of whole 16-byte units, no
 // reservoir) is taken from 3 x 2^20 FP32 nodes, where its prefetched rows read
 // HBM without stalls, and from 2^18 nodes where its blocks (30 columns by 8
-// rows, eight resident per SM) make one wave, which they fill; between the two
-// its long blocks leave part of a last wave empty, and the tiles win.
+// rows, eight resident per SM) make one wave: there it is ahead or level
+// (tiles / march: 480x560 28.6 / 27.6, 600x440 27.5 / 27.6, 1000x270 29.2 / 27.5,
+// 300x900 30.1 / 29.0, 2100x128 28.0 / 27.4, 540x512 29.5 / 27.8, 256x1024 27.5 /
+// 27.7; from a flushed L2 512x512 36.8 / 34.8), below it leaves SMs idle (500x500 26.5 / 27.7, 448x512 22.9 / 27.5), and
+// between the two lines its long blocks leave part of a last wave empty.
 // Everything else runs on tiles.  Up to two 32-node tiles per SM the lattice is
-// bound by one tile's latency and the tiles are split by lattice (split / best other tile: FP64 256x4 20.0 / 40.1, capillary 17.5 /
-// 34.1, 96x96 27.5 / 40.4, 128x128 52.2 / 44.0; FP32 64x40 4.9 / 5.5, 96x96
-// 5.1 / 6.5, 128x128 7.4 / 6.0); above that 32 x 4 in FP32 (whole lines) and
-// 16 x 8 in FP64 (bound by operations, so the smaller halo counts).  Lattices
+// bound by one tile's latency and the tiles are split by lattice (split / best
+// other tile: FP64 256x4 20.0 / 40.1, capillary 17.5 / 34.1, 96x96 27.5 / 40.4,
+// 128x128 52.2 / 44.0; FP32 64x40 4.9 / 5.5, 96x96 5.1 / 6.5, 128x128 7.4 / 6.0;
+// six species 128x64 FP64 67.7 / 99.0, FP32 7.7 / 8.4, 128x128 123 / 98, 13.4 /
+// 8.5); above that 32 x 4 in FP32 (whole lines) and
+// 16 x 8 in FP64 (bound by operations, so the smaller halo counts; six species
+// 512x512 1047 against 1064 in 32 x 4 and 1162 in two passes).  Lattices
 // of one or two rows would leave most of a tile idle and take the two-pass
 // form once they fill the GPU, and so do lattices with more rows than the tiles'
 // grids can count.

@@ -10,7 +10,8 @@
 // kernel parameter that points to such memory is not declared restrict (a
 // read-only load of it could be moved above the wait).
 //
-// Per step, plain -> dependent launches: 64 x 40 FP32 5.1 -> 3.6 us, 512 x 384
+// Per step of short runs (10 to 100 steps and the read of the populations), plain ->
+// dependent launches: 64 x 40 FP32 5.1 -> 3.6 us, 512 x 384
 // with reservoirs 28.8 -> 26.7, 701 x 523 with walls 50.1 -> 47.1, 512 x 512
 // 33.0 -> 30.4, adjoint 256 x 256 (each of 20 steps) 128 -> 112; 2048 x 2048
 // unchanged.  Not used where a kernel lives on the L1 cache behind one that

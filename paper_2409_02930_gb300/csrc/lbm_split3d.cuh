@@ -67,8 +67,8 @@ constexpr size_t split_smem_bytes(int NB, bool collide, bool park) {
 // 48 nodes in blocks of 32 ran 16 warps on two SMs, in blocks of 8 four warps on
 // each of six.  Larger lattices lose, since more warps carry the same nodes.
 // us per step with 32 / 16 / 8 nodes in a block: 12 x 2 x 2 88 / 63 / 56, 512
-// nodes 85 / 61 / 54, 1,024 85 / 61 / 74, 4,096 152 / 123 / 137, 8,192 153 / 201 /
-// 238; reactive 12 x 2 x 2 141 / 115 / 107.  FP32 gains nothing (12 x 2 x 2 9.5 /
+// nodes 85 / 61 / 54, 1,024 85 / 61 / 74, 4,096 152 / 123 / 137, 4,864 153 / 126,
+// 5,120 153 / 162, 8,192 153 / 201 / 238; reactive 12 x 2 x 2 141 / 115 / 107.  FP32 gains nothing (12 x 2 x 2 9.5 /
 // 10.1 / 9.4, 4,096 nodes 12.9 / 13.4 / 16.8).
 constexpr int split3d_nodes8 = 152 * 4, split3d_nodes16 = 152 * 32;
 

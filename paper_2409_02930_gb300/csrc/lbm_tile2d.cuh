@@ -17,9 +17,9 @@
 // a bare copy of the state 14.0 us, pulls and halo without arithmetic 20.7 us,
 // the step 30.4 us at 12 warps per SM; 128 registers and 16 warps, 256-node
 // blocks, and two nodes per thread in packed FP32 arithmetic were no faster);
-// in FP64 the FP64 pipe.  Against the form that served each size before:
-// 512 x 384 FP32 with reservoirs 158 -> 24.9 us per step, 701 x 523 with walls
-// 73 -> 44, 512 x 512 FP64 1010 -> 536.  Lattices of a few thousand nodes are
+// in FP64 the FP64 pipe.  Against the form that served each size before, us per
+// step of long runs: 512 x 384 FP32 with reservoirs 148 -> 21.9, 701 x 523 with
+// walls 65 -> 41, 512 x 512 FP64 974 -> 533.  Lattices of a few thousand nodes are
 // bound by one block's latency and run split by lattice (lbm_split2d.cuh).
 #pragma once
 
